@@ -165,7 +165,8 @@ typedef struct {
     int64_t sweeps;        /* productive Jacobi sweeps of the last kz_kernelize */
     int64_t passes;        /* rule evaluations over the whole graph, the certifying one included */
     int64_t edge_tests;    /* live edges tested, summed over passes */
-    int32_t path;          /* kz_path that ran */
+    int32_t path;          /* kz_path that ran; under KZ_PATH_AUTO, KZ_PATH_TENSOR also stands for the
+                              pair-by-pair passes that AUTO runs in the tensor form's region */
     int32_t status;        /* kz_status recorded on the device by the last kz_kernelize */
     int32_t k;             /* colours */
     int32_t clique_k;      /* clique size q the last kz_kernelize used */

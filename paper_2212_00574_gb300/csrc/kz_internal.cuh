@@ -146,6 +146,7 @@ struct kz_graph_s {
   float learned_threshold = 0.5f;
   void *learned_bufs = nullptr;
   void *tensor_bufs = nullptr;  // tensor-core path scratch
+  void *pairs_bufs = nullptr;   // pair form scratch
   void *support_bufs = nullptr; // per-class support counts (CSR path, support schedule)
   void *dominance_bufs = nullptr;  // vertex dominance rounds
   int32_t dom_rounds = 0;          // dominance rounds of the last kz_kernelize that deleted something
@@ -207,6 +208,16 @@ kz_status tensor_kernelize(kz_graph g, const kz_options &opt, cudaStream_t s);
 // when it deleted something and the run may go on.
 kz_status tensor_one_pass(kz_graph g, const kz_options &opt, cudaStream_t s, int *cont);
 void tensor_release(kz_graph g);
+
+// Pair form of the passes (kz_pairs.cu): what AUTO runs in the tensor form's
+// region.  pairs_one_pass is to tensor_one_pass as pairs_kernelize is to
+// tensor_kernelize.
+kz_status pairs_kernelize(kz_graph g, const kz_options &opt, cudaStream_t s);
+kz_status pairs_one_pass(kz_graph g, cudaStream_t s, int *cont);
+void pairs_release(kz_graph g);
+// Full passes of the learned and support schedules: KZ_PATH_BITSET,
+// KZ_PATH_TENSOR or this value.
+constexpr int kFullPairs = 64;
 // The driver's cuTensorMapEncodeTiled, found through the runtime's entry-point
 // query (null when the driver does not provide it).
 void *tensor_map_encoder();

@@ -1141,8 +1141,15 @@ struct RunEvents {
   }
 };
 
-// Learned schedule (see the file comment).  full_path is the path of the
-// full passes: KZ_PATH_BITSET (the multi-CTA sweep) or KZ_PATH_TENSOR.
+// One full pass on the path the schedule was given: KZ_PATH_BITSET (the
+// multi-CTA sweep), KZ_PATH_TENSOR or kFullPairs (the pair form).
+static kz_status run_full_pass(kz_graph g, const kz_options &opt, int full_path, cudaStream_t s, int *cont) {
+  if (full_path == kFullPairs) return pairs_one_pass(g, s, cont);
+  if (full_path == KZ_PATH_TENSOR) return tensor_one_pass(g, opt, s, cont);
+  return bitset_one_pass(g, s, cont);
+}
+
+// Learned schedule (see the file comment); full_path as run_full_pass.
 kz_status learned_kernelize(kz_graph g, const kz_options &opt, int full_path, cudaStream_t s) {
   if (!g->model) return KZ_ERR_UNSUPPORTED;
   if (!g->learned_bufs) {
@@ -1171,7 +1178,7 @@ kz_status learned_kernelize(kz_graph g, const kz_options &opt, int full_path, cu
   bool calibrated = false;
   auto full_pass = [&](int *cont) -> kz_status {
     KZ_CUDA_TRY(cudaEventRecord(ev.a, s));
-    const kz_status st = full_path == KZ_PATH_TENSOR ? tensor_one_pass(g, opt, s, cont) : bitset_one_pass(g, s, cont);
+    const kz_status st = run_full_pass(g, opt, full_path, s, cont);
     KZ_CUDA_TRY(cudaEventRecord(ev.b, s));
     KZ_CUDA_TRY(cudaEventSynchronize(ev.b));
     const double ms = ev.ms();
@@ -1410,7 +1417,7 @@ kz_status recheck_kernelize(kz_graph g, const kz_options &opt, int full_path, cu
   // a full pass, timed; then its deletions listed from the two buffers
   auto full_sweep = [&](int *cont) -> kz_status {
     KZ_CUDA_TRY(cudaEventRecord(ev.a, s));
-    KZ_TRY(full_path == KZ_PATH_TENSOR ? tensor_one_pass(g, opt, s, cont) : bitset_one_pass(g, s, cont));
+    KZ_TRY(run_full_pass(g, opt, full_path, s, cont));
     KZ_CUDA_TRY(cudaEventRecord(ev.b, s));
     KZ_CUDA_TRY(cudaEventSynchronize(ev.b));
     const double ms = ev.ms();
