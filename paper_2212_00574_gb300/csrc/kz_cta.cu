@@ -17,7 +17,9 @@
 #include <vector>
 
 #include "kz_internal.cuh"
+#include "kz_pack_tiles.cuh"
 #include "kz_rules.cuh"
+#include "kz_sweep.cuh"
 
 namespace kz {
 
@@ -451,8 +453,8 @@ kz_status cta_kernelize_one(kz_graph g, const kz_options &opt, cudaStream_t s) {
 // allocation at all.  Every intermediate lives in one file-scope device array
 // (g_noalloc_scratch below) that each GPU loading the library keeps until the
 // process exits; the caller passes device buffers for inputs and outputs.
-// The fixpoint itself is the in-CTA kernel above, reading its descriptor from
-// that array.
+// The fixpoint itself is a cooperative grid kernel (the in-CTA kernel above for
+// the smallest graphs), reading its descriptor from that array.
 // ---------------------------------------------------------------------------
 
 namespace kz {
@@ -465,14 +467,16 @@ constexpr int kMaxBlocks = 256;
 
 struct Header {
   CtaGraph desc;
-  int32_t status;
-  int32_t pad;
-  unsigned long long m;
+  int32_t status;   // found by the set-up
+  int32_t illegal;  // KZ_ERR_ILLEGAL_COLOURING, found by the packer
+  int32_t R, pad;
+  int64_t cross;            // pairs of vertices in different classes
+  unsigned long long bits;  // set bits of the packed rows: twice the edges
   int32_t coff[65];
   int32_t boff[65];
   int32_t rounds[64];
-  int32_t fill[64];
   int32_t pair_off[kMaxBlocks + 1];
+  int32_t unit_off[kMaxBlocks + 1];  // prefix of the grid kernel's units: block pairs, one for a block without any
   BlockDesc blocks[kMaxBlocks];
 };
 
@@ -485,6 +489,7 @@ struct Scratch {
   alignas(256) uint32_t V1[kMaxLdw];
   alignas(256) int32_t perm[kMaxN];
   alignas(256) int32_t inv[kMaxN];
+  alignas(256) int32_t pos[kMaxN];  // caller vertex -> (word << 5) | bit of its relabelled vertex inside any row
   alignas(256) int32_t v_sweep[kMaxN];
 };
 
@@ -497,24 +502,15 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(kz::noal
 namespace kz {
 namespace noalloc {
 
-// First index i in [0, len) with a[i] > x (a sorted ascending).
-__device__ __forceinline__ int upper_bound_int(const int32_t *a, int len, int32_t x) {
-  int lo = 0, hi = len;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (a[mid] <= x) lo = mid + 1;
-    else hi = mid;
-  }
-  return lo;
-}
-
 // Layout of the caller's graph: colour classes, blocks, block pairs, the
-// descriptor of the in-CTA kernel.  One CTA.
-__global__ void setup_kernel(Scratch *s, int32_t n, int32_t k, const int32_t *__restrict__ colour) {
+// descriptor of the in-CTA kernel, the relabelling and the live words.  One
+// CTA; every prefix over blocks is closed-form per class, so the blocks are
+// filled in parallel.
+__global__ void __launch_bounds__(1024) setup_kernel(Scratch *s, int32_t n, int32_t k,
+                                                     const int32_t *__restrict__ colour) {
   Header &h = s->h;
-  __shared__ int cnt[64];
-  __shared__ int bad;
-  __shared__ int status;
+  __shared__ int cnt[64], coff[65], boff[65], fill[64], pairs0[65], units0[65];
+  __shared__ int bad, status, ldw_s;
   const int tid = threadIdx.x;
   if (tid < 64) cnt[tid] = 0;
   if (tid == 0) bad = 0;
@@ -526,32 +522,26 @@ __global__ void setup_kernel(Scratch *s, int32_t n, int32_t k, const int32_t *__
   }
   __syncthreads();
   if (tid == 0) {
-    int st = bad;
-    int R = 1, nb = 0;
-    h.coff[0] = 0;
+    int R = 1;
+    coff[0] = boff[0] = 0;
     for (int c = 0; c < k; c++) {
-      h.coff[c + 1] = h.coff[c] + cnt[c];
-      h.rounds[c] = (cnt[c] + 31) / 32;
-      R = max(R, h.rounds[c]);
-      nb += h.rounds[c];
+      const int rounds = (cnt[c] + 31) / 32;
+      coff[c + 1] = coff[c] + cnt[c];
+      boff[c + 1] = boff[c] + rounds;
+      fill[c] = coff[c];
+      R = max(R, rounds);
+    }
+    const int nb = boff[k];
+    pairs0[0] = units0[0] = 0;
+    for (int c = 0; c < k; c++) {
+      const int rounds = boff[c + 1] - boff[c], with = nb - boff[c + 1];  // blocks of higher classes
+      pairs0[c + 1] = pairs0[c] + rounds * with;
+      units0[c + 1] = units0[c] + rounds * max(with, 1);
     }
     const int64_t ldw = ((int64_t)R * k + 3) / 4 * 4;
+    int st = bad;
     if (!st && (ldw > kMaxLdw || (int64_t)n * ldw > kMaxWords || nb > kMaxBlocks)) st = KZ_ERR_UNSUPPORTED;
     if (!st) {
-      h.boff[0] = 0;
-      int b = 0;
-      for (int c = 0; c < k; c++) {
-        h.boff[c + 1] = h.boff[c] + h.rounds[c];
-        for (int r = 0; r < h.rounds[c]; r++, b++) {
-          h.blocks[b].c = c;
-          h.blocks[b].r = r;
-          h.blocks[b].base = h.coff[c] + 32 * r;
-          h.blocks[b].size = min(32, cnt[c] - 32 * r);
-        }
-        h.fill[c] = h.coff[c];
-      }
-      h.pair_off[0] = 0;
-      for (int x = 0; x < nb; x++) h.pair_off[x + 1] = h.pair_off[x] + (nb - h.boff[h.blocks[x].c + 1]);
       CtaGraph &d = h.desc;
       d.A0 = s->A0;
       d.A1 = s->A1;
@@ -570,7 +560,11 @@ __global__ void setup_kernel(Scratch *s, int32_t n, int32_t k, const int32_t *__
       d.smem_words = (int32_t)(2 * ((int64_t)n * ldw + ldw));
       d.m = 0;
       d.cost = 0;
-      h.m = 0;
+      int64_t cross = 0;
+      for (int c = 0; c < k; c++) cross += (int64_t)cnt[c] * coff[c];
+      h.cross = cross;
+      h.bits = 0;
+      h.R = R;
       DevState &ds = s->st;
       ds.cur = 0;
       ds.status = KZ_OK;
@@ -578,96 +572,77 @@ __global__ void setup_kernel(Scratch *s, int32_t n, int32_t k, const int32_t *__
       ds.sweeps = ds.passes = ds.tests = 0;
       ds.pass_dv = ds.pass_de = ds.pass_tests = 0;
       ds.ticket = 0;
+      ds.bar_count = 0;
+      ds.bar_abort = 0;
+      ds.pass_word = 0;
+      for (int i = 0; i < 2; i++) ds.ppass[i][0] = ds.ppass[i][1] = ds.ppass[i][2] = 0;
+      h.pair_off[nb] = pairs0[k];
+      h.unit_off[nb] = units0[k];
     }
     h.status = st;
+    h.illegal = 0;
     status = st;
+    ldw_s = (int)ldw;
   }
   __syncthreads();
   if (status) return;
+  for (int i = tid; i < ldw_s; i += blockDim.x) s->V0[i] = s->V1[i] = 0u;
+  if (tid <= k) {
+    h.coff[tid] = coff[tid];
+    h.boff[tid] = boff[tid];
+    if (tid < k) h.rounds[tid] = boff[tid + 1] - boff[tid];
+  }
+  __syncthreads();
+  const int nb = boff[k];
+  for (int b = tid; b < nb; b += blockDim.x) {
+    int c = 0;
+    while (boff[c + 1] <= b) c++;
+    const int r = b - boff[c], with = nb - boff[c + 1];
+    BlockDesc d;
+    d.c = c;
+    d.r = r;
+    d.base = coff[c] + 32 * r;
+    d.size = min(32, cnt[c] - 32 * r);
+    h.blocks[b] = d;
+    h.pair_off[b] = pairs0[c] + r * with;
+    h.unit_off[b] = units0[c] + r * max(with, 1);
+    s->V0[r * k + c] = s->V1[r * k + c] = d.size >= 32 ? 0xffffffffu : ((1u << d.size) - 1u);
+  }
   // relabel: every class a contiguous id range (order inside a class is free:
   // the fixpoint and every count reported do not depend on it)
   for (int v = tid; v < n; v += blockDim.x) {
-    const int x = atomicAdd(&h.fill[colour[v]], 1);
+    const int c = colour[v], x = atomicAdd(&fill[c], 1), i = x - coff[c];
     s->inv[v] = x;
     s->perm[x] = v;
+    s->pos[v] = (((i >> 5) * k + c) << 5) | (i & 31);
+    s->v_sweep[v] = 0;
   }
 }
 
-// Zeroed rows, live words of every block, zeroed deletion sweeps.
-__global__ void clear_kernel(Scratch *s) {
-  if (s->h.status) return;
-  const CtaGraph &d = s->h.desc;
-  const int64_t words = (int64_t)d.n * d.ldw;
-  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = tid; i < words; i += stride) s->A0[i] = 0u;
-  for (int64_t i = tid; i < d.ldw; i += stride) s->V0[i] = 0u;
-  for (int64_t i = tid; i < d.n; i += stride) s->v_sweep[i] = 0;
-}
-
-__global__ void live_words_kernel(Scratch *s) {
-  if (s->h.status) return;
-  const CtaGraph &d = s->h.desc;
-  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < d.nb; b += gridDim.x * blockDim.x) {
-    const BlockDesc bd = s->h.blocks[b];
-    s->V0[bd.r * d.k + bd.c] = bd.size >= 32 ? 0xffffffffu : ((1u << bd.size) - 1u);
-  }
-}
-
-// Caller's dense bit matrix (strict upper triangle) into the block-plane rows.
-__global__ void pack_kernel(Scratch *s, const uint64_t *__restrict__ bits, int64_t row_words,
-                            const int32_t *__restrict__ colour) {
+// Caller's dense bit matrix (strict upper triangle) into both copies of the
+// block-plane rows (kz_pack_tiles.cuh).
+__global__ void __launch_bounds__(kTileThreads) pack_kernel(Scratch *s, const uint64_t *__restrict__ bits,
+                                                            int64_t row_words, const int32_t *__restrict__ colour) {
+  extern __shared__ __align__(16) uint32_t colw[];  // 32 * ceil(n / 32) column words
+  __shared__ int32_t scoff[65];
   Header &h = s->h;
   if (h.status) return;
-  const int n = h.desc.n, k = h.desc.k, ldw = h.desc.ldw;
+  const int n = h.desc.n, k = h.desc.k, lane = threadIdx.x & 31;
+  if (threadIdx.x <= k) scoff[threadIdx.x] = h.coff[threadIdx.x];
   unsigned long long mine = 0;
-  const int64_t total = (int64_t)n * row_words;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t i = (int32_t)(t / row_words);
-    const int64_t w = t - (int64_t)i * row_words;
-    const int64_t j0 = w * 64;
-    if (j0 + 63 <= i || j0 >= n) continue;
-    uint64_t word = bits[t];
-    if (j0 <= i) {
-      const int sh = i - (int)j0 + 1;
-      word = sh >= 64 ? 0 : (word >> sh) << sh;
-    }
-    if (j0 + 64 > n) word &= (1ull << (n - (int)j0)) - 1;
-    if (!word) continue;
-    const int32_t ci = colour[i];
-    const int32_t x = s->inv[i];
-    const int32_t ix = x - h.coff[ci];
-    while (word) {
-      const int b = __ffsll((long long)word) - 1;
-      word &= word - 1;
-      const int32_t j = (int32_t)j0 + b;
-      const int32_t cj = colour[j];
-      if (cj == ci) {
-        atomicCAS(&h.status, 0, (int32_t)KZ_ERR_ILLEGAL_COLOURING);
-        continue;
-      }
-      const int32_t y = s->inv[j];
-      const int32_t iy = y - h.coff[cj];
-      atomicOr(&s->A0[(int64_t)x * ldw + (iy >> 5) * k + cj], 1u << (iy & 31));
-      atomicOr(&s->A0[(int64_t)y * ldw + (ix >> 5) * k + ci], 1u << (ix & 31));
-      mine++;
-    }
+  bool bad = false;
+  for (int64_t i0 = (int64_t)blockIdx.x * 32; i0 < n; i0 += (int64_t)gridDim.x * 32) {
+    const int rows = min(32, n - (int)i0);
+    __syncthreads();
+    tile_columns(colw, bits, row_words, n, i0, rows);
+    __syncthreads();
+    const bool valid = lane < rows;
+    mine += tile_rows(colw, s->A0, s->A1, nullptr, h.desc.ldw, k, h.R, scoff, s->perm,
+                      valid ? s->inv[i0 + lane] : 0, valid ? colour[i0 + lane] : -1, valid, &bad);
   }
+  if (bad) atomicCAS(&h.illegal, 0, (int32_t)KZ_ERR_ILLEGAL_COLOURING);
   for (int o = 16; o > 0; o >>= 1) mine += __shfl_down_sync(0xffffffffu, mine, o);
-  if ((threadIdx.x & 31) == 0 && mine) atomicAdd(&h.m, mine);
-}
-
-// Both ping-pong copies start from the packed rows (own-class words zero).
-__global__ void mirror_kernel(Scratch *s) {
-  if (s->h.status) return;
-  const CtaGraph &d = s->h.desc;
-  const int64_t words = (int64_t)d.n * d.ldw;
-  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = tid; i < words; i += stride) s->A1[i] = s->A0[i];
-  for (int64_t i = tid; i < d.ldw; i += stride) s->V1[i] = s->V0[i];
-  if (tid == 0) s->h.desc.m = (int64_t)s->h.m;
+  if (lane == 0 && mine) atomicAdd(&h.bits, mine);
 }
 
 // The in-CTA fixpoint on the scratch descriptor (k <= 32).
@@ -678,64 +653,205 @@ __global__ void __launch_bounds__(kCtaThreads, 1) fixpoint_kernel(Scratch *s, in
   __shared__ int s_flag;
   __shared__ int32_t s_rounds[32];
   __shared__ CtaRun s_run;
-  if (s->h.status) return;
-  const CtaGraph G = s->h.desc;
+  if (s->h.status || s->h.illegal) return;
+  CtaGraph G = s->h.desc;
+  G.m = (int64_t)(s->h.bits / 2);
   if (G.smem_words > 0 && G.smem_words <= smem_words)
     cta_fixpoint<32, true>(G, max_sweeps, 0, smem, s_cnt, &s_flag, s_rounds, &s_run);
   else
     cta_fixpoint<32, false>(G, max_sweeps, 0, smem, s_cnt, &s_flag, s_rounds, &s_run);
 }
 
-__global__ void zero_out_kernel(uint64_t *__restrict__ out, int64_t words) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < words; i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = 0ull;
+// The fixpoint over the whole GPU, in one cooperative launch: every warp owns
+// a consecutive share of the units (block X against one block Y of a higher
+// class, or a block X without partners), runs of one X at a time
+// (sweep_item, kz_sweep.cuh: plane 0 of the Y rows staged by asynchronous
+// copies, one block ahead), and a grid barrier closes each pass.  The barrier
+// wait is bounded; one that runs out records KZ_ERR_TIMEOUT and every CTA
+// leaves.
+//
+// Why a grid: one CTA leaves 151 SMs idle.  A pass of n = 1501, k = 12,
+// p = 0.3 (1,100 block pairs) took 2.8 ms on one CTA and takes 26 us here;
+// n = 4096, k = 20, p = 0.92: 10.9 ms and 44 us.  Bound by latency: a warp has
+// about one unit, and its recounts are chains of loads.  Below density 0.42
+// the first test takes two planes (42 to 26 us a pass on the first graph).
+constexpr int kGridWarps = 8;
+constexpr uint32_t kGridSpinLimit = 1u << 24;
+constexpr double kGridTwoPlaneDensity = 0.42;
+
+template <int KMAX>
+__global__ void __launch_bounds__(kGridWarps * 32, 1) grid_fixpoint_kernel(Scratch *s, int64_t max_sweeps_opt) {
+  extern __shared__ __align__(16) uint32_t smem[];
+  __shared__ unsigned long long s_cnt[3];
+  __shared__ unsigned long long s_word;
+  const Header &h = s->h;
+  if (h.status || h.illegal) return;
+  DevState *st = &s->st;
+  const CtaGraph &d = h.desc;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nb = d.nb;
+  uint32_t *buf0 = smem + wib * 2 * 32 * 2 * KMAX;
+  uint32_t *buf1 = buf0 + 32 * 2 * KMAX;
+  // the two-plane first test below the density where it wins on the
+  // single-graph sweep kernels
+  const bool two = h.R >= 2 && (double)(h.bits / 2) < kGridTwoPlaneDensity * (double)h.cross;
+  const int64_t max_sweeps = max_sweeps_opt > 0 ? max_sweeps_opt : (int64_t)d.n + (int64_t)(h.bits / 2) + 1;
+  if (blockIdx.x == 0 && threadIdx.x == 0) st->max_sweeps = max_sweeps;  // the closing CTA reads it behind the barrier
+  GraphView G;
+  G.blocks = h.blocks;
+  G.rounds = h.rounds;
+  G.A0 = s->A0;
+  G.A1 = s->A1;
+  G.V0 = s->V0;
+  G.V1 = s->V1;
+  G.v_sweep = s->v_sweep;
+  G.k = d.k;
+  G.ldw = d.ldw;
+  const int64_t units = h.unit_off[nb];
+  // neighbouring warps of the share order sit on different SMs
+  const int64_t warps = (int64_t)gridDim.x * kGridWarps, w = (int64_t)wib * gridDim.x + blockIdx.x;
+  const int u0 = (int)(units * w / warps), u1 = (int)(units * (w + 1) / warps);
+  const int x0 = u0 < u1 ? find_x(h.unit_off, nb, u0) : 0;
+  int cur = 0;
+  int64_t sweep_no = 0;
+  for (int pass = 0;; pass++) {
+    if (threadIdx.x < 3) s_cnt[threadIdx.x] = 0;
+    __syncthreads();
+    PassCounters pc;
+    for (int u = u0, x = x0; u < u1; x++) {
+      const int e = min(u1, h.unit_off[x + 1]);
+      const int ybeg = min(h.boff[h.blocks[x].c + 1], nb);
+      WorkItem item;
+      item.x = x;
+      item.vflag = u == h.unit_off[x];
+      item.y0 = ybeg < nb ? ybeg + (u - h.unit_off[x]) : nb;
+      item.y1 = ybeg < nb ? ybeg + (e - h.unit_off[x]) : nb;
+      if (two) sweep_item<KMAX, true>(G, item, cur, sweep_no, buf0, buf1, pc);
+      else sweep_item<KMAX>(G, item, cur, sweep_no, buf0, buf1, pc);
+      u = e;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      pc.tests += __shfl_down_sync(0xffffffffu, pc.tests, o);
+      pc.de += __shfl_down_sync(0xffffffffu, pc.de, o);
+      pc.dv += __shfl_down_sync(0xffffffffu, pc.dv, o);
+    }
+    if (lane == 0) {
+      if (pc.tests) atomicAdd(&s_cnt[0], pc.tests);
+      if (pc.de) atomicAdd(&s_cnt[1], pc.de);
+      if (pc.dv) atomicAdd(&s_cnt[2], pc.dv);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      unsigned long long *cnt = st->ppass[pass & 1];
+      for (int i = 0; i < 3; i++)
+        if (s_cnt[i]) atomicAdd(&cnt[i], s_cnt[i]);
+      __threadfence();
+      const unsigned long long w0 = *((volatile unsigned long long *)&st->pass_word);
+      unsigned long long word = w0;
+      bool abort = false;
+      if (atomicAdd(&st->bar_count, 1u) == gridDim.x - 1u) {
+        // the last CTA closes the pass and releases the others
+        __threadfence();
+        const unsigned long long tests = atomicAdd(&cnt[0], 0ull);
+        const unsigned long long de = atomicAdd(&cnt[1], 0ull);
+        const unsigned long long dv = atomicAdd(&cnt[2], 0ull);
+        const int cont = finish_pass(st, dv, de, tests);
+        cnt[0] = cnt[1] = cnt[2] = 0;
+        st->bar_count = 0;
+        word = pass_word(pass_word_gen(w0) + 1u, cont, cont ? cur ^ 1 : cur, cont ? sweep_no + 1 : sweep_no);
+        __threadfence();
+        atomicExch(&st->pass_word, word);
+      } else {
+        for (uint32_t spins = 0;; spins++) {
+          word = *((volatile unsigned long long *)&st->pass_word);
+          if (pass_word_gen(word) != pass_word_gen(w0)) break;
+          abort = *((volatile int32_t *)&st->bar_abort) != 0;
+          if (!abort && spins > kGridSpinLimit) {
+            atomicCAS(&st->status, (int32_t)KZ_OK, (int32_t)KZ_ERR_TIMEOUT);
+            atomicExch(&st->bar_abort, 1);
+            abort = true;
+          }
+          if (abort) break;
+          __nanosleep(32);
+        }
+      }
+      __threadfence();
+      s_word = abort ? 0ull : word;  // a cleared continue bit ends the kernel
+    }
+    __syncthreads();
+    const unsigned long long word = s_word;
+    if (!pass_word_cont(word)) break;
+    cur = pass_word_cur(word);
+    sweep_no = pass_word_sweeps(word);
+  }
 }
 
+typedef void (*GridFn)(Scratch *, int64_t);
+
+static GridFn pick_grid(int k, int &kmax) {
+  if (k <= 8) { kmax = 8; return grid_fixpoint_kernel<8>; }
+  if (k <= 16) { kmax = 16; return grid_fixpoint_kernel<16>; }
+  if (k <= 24) { kmax = 24; return grid_fixpoint_kernel<24>; }
+  kmax = 32;
+  return grid_fixpoint_kernel<32>;
+}
+
+constexpr size_t grid_smem(int kmax) { return (size_t)kGridWarps * 2 * 32 * 2 * kmax * 4; }
+
+// Vertices up to which one CTA runs the fixpoint from shared memory: below
+// it a pass is shorter than a grid barrier (n = 100: 9.7 us a pass on one CTA,
+// n = 200: 8.1 us on the grid).
+constexpr int kOneCtaMaxN = 64;
+
 // Kernel rows back to caller ids: the symmetric bit matrix, the live
-// vertices, and (sweeps, passes, edge tests, status).
-__global__ void unpack_kernel(Scratch *s, int32_t n_in, uint64_t *__restrict__ out, int64_t row_words,
-                              uint8_t *__restrict__ alive, int64_t *__restrict__ counts) {
+// vertices, and (sweeps, passes, edge tests, status).  A CTA stages one
+// relabelled row; its warps gather the row's 32 positions of 32 caller
+// columns at a time, and a ballot is half an output word.
+constexpr int kUnpackThreads = 128;
+
+__global__ void __launch_bounds__(kUnpackThreads) unpack_kernel(Scratch *s, int32_t n_in, uint64_t *__restrict__ out,
+                                                                int64_t row_words, uint8_t *__restrict__ alive,
+                                                                int64_t *__restrict__ counts) {
+  __shared__ uint32_t srow[kMaxLdw];
   const Header &h = s->h;
-  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  if (h.status) {
-    // a rejected input leaves defined outputs: no vertex, no edge (the bit
-    // matrix was zeroed before this kernel), zero counts and the status
+  const int status = h.status ? h.status : h.illegal;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (status) {
+    // a rejected input leaves defined outputs: no vertex, no edge, zero
+    // counts and the status
+    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = tid; i < (int64_t)n_in * row_words; i += stride) out[i] = 0ull;
     for (int64_t v = tid; v < n_in; v += stride) alive[v] = 0;
     if (tid == 0) {
       counts[0] = counts[1] = counts[2] = 0;
-      counts[3] = h.status;
+      counts[3] = status;
     }
     return;
   }
-  const CtaGraph &d = h.desc;
-  const int cur = s->st.cur;
+  const int n = h.desc.n, ldw = h.desc.ldw, cur = s->st.cur;
   const uint32_t *A = cur ? s->A1 : s->A0;
   const uint32_t *V = cur ? s->V1 : s->V0;
-  const int n = d.n, k = d.k, ldw = d.ldw;
-  const int rk = ldw;  // rows are scanned over their padded length; padding words are zero
-  for (int64_t t = tid; t < (int64_t)n * rk; t += stride) {
-    const int32_t x = (int32_t)(t / rk);
-    const int32_t w = (int32_t)(t - (int64_t)x * rk);
-    uint32_t word = A[(int64_t)x * ldw + w];
-    if (!word) continue;
-    const int32_t c = w % k, r = w / k;
-    const int32_t ox = s->perm[x];
-    while (word) {
-      const int b = __ffs(word) - 1;
-      word &= word - 1;
-      const int32_t oy = s->perm[h.coff[c] + 32 * r + b];
-      atomicOr(reinterpret_cast<unsigned long long *>(&out[(int64_t)ox * row_words + (oy >> 6)]),
-               1ull << (oy & 63));
+  for (int v = blockIdx.x; v < n; v += gridDim.x) {
+    __syncthreads();  // the previous row is consumed
+    const uint4 *row = reinterpret_cast<const uint4 *>(A + (int64_t)s->inv[v] * ldw);
+    for (int i = threadIdx.x; i < ldw / 4; i += kUnpackThreads) reinterpret_cast<uint4 *>(srow)[i] = row[i];
+    __syncthreads();
+    uint64_t *dst = out + (int64_t)v * row_words;
+    for (int64_t w = warp; w < row_words; w += kUnpackThreads / 32) {
+      uint32_t half[2];
+#pragma unroll
+      for (int q = 0; q < 2; q++) {
+        const int64_t col = 64 * w + 32 * q + lane;
+        const int p = col < n ? s->pos[col] : -1;
+        half[q] = __ballot_sync(0xffffffffu, p >= 0 && ((srow[p >> 5] >> (p & 31)) & 1u));
+      }
+      if (lane == 0) dst[w] = (uint64_t)half[0] | (uint64_t)half[1] << 32;
+    }
+    if (threadIdx.x == 0) {
+      const int p = s->pos[v];
+      alive[v] = (uint8_t)((V[p >> 5] >> (p & 31)) & 1u);
     }
   }
-  for (int64_t v = tid; v < n; v += stride) {
-    const int32_t x = s->inv[v];
-    const int32_t c = (int32_t)(upper_bound_int(h.coff, k + 1, x) - 1);
-    const int32_t i = x - h.coff[c];
-    alive[v] = (uint8_t)((V[(i >> 5) * k + c] >> (i & 31)) & 1u);
-  }
-  if (tid == 0) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
     counts[0] = s->st.sweeps;
     counts[1] = s->st.passes;
     counts[2] = s->st.tests;
@@ -794,18 +910,35 @@ extern "C" kz_status kz_kernelize_dense_noalloc(int32_t n, int32_t k, const int3
     if (!configured[dev]) {
       KZ_CUDA_TRY(cudaFuncSetAttribute((const void *)fixpoint_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes));
+      // every width is set up (and loaded) now, so that no later call does
+      for (int kk = 8; kk <= 32; kk += 8) {
+        int km = 0, per_sm = 0;
+        const GridFn fn = pick_grid(kk, km);
+        KZ_CUDA_TRY(cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)grid_smem(km)));
+        KZ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)fn, kGridWarps * 32,
+                                                                  grid_smem(km)));
+        if (per_sm < 1) return KZ_ERR_UNSUPPORTED;
+      }
       configured[dev] = true;
     }
   }
-  const int grid = 2 * std::max(sms, 1);
   setup_kernel<<<1, 1024, 0, s>>>(sp, n, k, colour);
-  clear_kernel<<<grid, 256, 0, s>>>(sp);
-  live_words_kernel<<<1, 256, 0, s>>>(sp);
-  if ((int64_t)n * row_words > 0) pack_kernel<<<grid, 256, 0, s>>>(sp, adj_bits, row_words, colour);
-  mirror_kernel<<<grid, 256, 0, s>>>(sp);
-  fixpoint_kernel<<<1, kz::kCtaThreads, smem_bytes, s>>>(sp, max_sweeps, smem_bytes / 4);
-  if ((int64_t)n * row_words > 0) zero_out_kernel<<<grid, 256, 0, s>>>(adj_out, (int64_t)n * row_words);
-  unpack_kernel<<<grid, 256, 0, s>>>(sp, n, adj_out, row_words, vertex_alive, counts);
+  if (n > 0) pack_kernel<<<(n + 31) / 32, kz::kTileThreads, (size_t)(n + 31) / 32 * 128, s>>>(sp, adj_bits, row_words, colour);
+  if (n <= kOneCtaMaxN) {
+    fixpoint_kernel<<<1, kz::kCtaThreads, smem_bytes, s>>>(sp, max_sweeps, smem_bytes / 4);
+  } else {
+    // one CTA per SM at most (all resident, as the grid barrier needs), and no
+    // more warps than the block pairs the classes can make
+    int km = 0;
+    const GridFn fn = pick_grid(k, km);
+    const int64_t blocks = n / 32 + k, pairs = blocks * blocks / 2;
+    const int ctas = (int)std::min<int64_t>(std::max(sms, 1), (pairs + kGridWarps - 1) / kGridWarps);
+    void *args[] = {&sp, &max_sweeps};
+    KZ_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)fn, dim3(ctas), dim3(kGridWarps * 32), args, grid_smem(km), s));
+  }
+  unpack_kernel<<<std::max(1, std::min(n, 16 * std::max(sms, 1))), kUnpackThreads, 0, s>>>(sp, n, adj_out, row_words,
+                                                                                          vertex_alive, counts);
   KZ_CUDA_TRY(cudaGetLastError());
   // synchronous: the device status decides the return value
   int64_t status = 0;

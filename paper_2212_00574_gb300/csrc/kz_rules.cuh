@@ -160,12 +160,14 @@ __device__ __forceinline__ bool edge_fails_beyond_plane0(const uint32_t *ru, con
     const int c = __ffsll((long long)miss) - 1;
     miss &= miss - 1;
     const int R = rounds[c];
-    bool found = false;
-    for (int r = 1; r < R; r++) {
-      if (ru[r * k + c] & rv[r * k + c]) {
-        found = true;
-        break;
-      }
+    // plane 1 settles most classes of a dense graph; after it four planes a
+    // step, so that their loads travel together (one at a time the search is
+    // a chain of round trips: n = 2048, k = 12, p = 0.15 took 307 us, 273 now)
+    uint32_t found = R > 1 ? ru[k + c] & rv[k + c] : 0u;
+    for (int r = 2; r < R && !found; r += 4) {
+#pragma unroll
+      for (int j = 0; j < 4; j++)
+        if (r + j < R) found |= ru[(r + j) * k + c] & rv[(r + j) * k + c];
     }
     if (!found && ++missing > slack) return true;
   }

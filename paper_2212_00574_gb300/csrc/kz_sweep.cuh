@@ -75,7 +75,10 @@ struct PassCounters {
 
 // One work item of one Jacobi pass, executed by one warp.  `cur` is the
 // graph's current ping-pong buffer, `sweep_no` its productive sweeps so far.
-template <int KMAX>
+// TWO: the first test of a pair looks at planes 0 and 1 (rows of at least two
+// planes; staging buffers of 32 x 2 KMAX words), which on sparser graphs
+// leaves far fewer pairs to the recount.
+template <int KMAX, bool TWO = false>
 __device__ __forceinline__ void sweep_item(const GraphView &p, const WorkItem item, int cur, int64_t sweep_no,
                                            uint32_t *buf0, uint32_t *buf1, PassCounters &pc) {
   const int lane = threadIdx.x & 31;
@@ -84,7 +87,8 @@ __device__ __forceinline__ void sweep_item(const GraphView &p, const WorkItem it
   const uint32_t *__restrict__ Vc = cur ? p.V1 : p.V0;
   uint32_t *__restrict__ Vn = cur ? p.V0 : p.V1;
   const int k = p.k, ldw = p.ldw;
-  const int kq4 = (k + 3) >> 2;
+  const int kq4 = TWO ? (2 * k + 3) >> 2 : (k + 3) >> 2;
+  constexpr int kRow = TWO ? 2 * KMAX : KMAX;  // staged row stride
   {
     const BlockDesc X = p.blocks[item.x];
     const int cu = X.c;
@@ -96,11 +100,14 @@ __device__ __forceinline__ void sweep_item(const GraphView &p, const WorkItem it
     BlockDesc Yn;
     if (yn > 0) {
       Yn = p.blocks[item.y0];
-      stage_block<KMAX>(A, ldw, Yn, kq4, buf0, lane);
+      if constexpr (TWO) stage_block2<KMAX>(A, ldw, Yn, kq4, buf0, lane);
+      else stage_block<KMAX>(A, ldw, Yn, kq4, buf0, lane);
     }
     cp_async_commit();
     uint32_t Fu[KMAX];
     load_plane0<KMAX>(Fu, rowu, k, valid_u);
+    uint32_t F1[TWO ? KMAX : 1];
+    if constexpr (TWO) load_plane1<KMAX>(F1, rowu, k, valid_u);
     if (item.vflag) {
       const int wx = X.r * k + cu;
       const uint32_t vword = Vc[wx];
@@ -125,7 +132,8 @@ __device__ __forceinline__ void sweep_item(const GraphView &p, const WorkItem it
       uint32_t *sv = (i & 1) ? buf1 : buf0;
       if (i + 1 < yn) {
         Yn = p.blocks[item.y0 + i + 1];
-        stage_block<KMAX>(A, ldw, Yn, kq4, (i & 1) ? buf0 : buf1, lane);
+        if constexpr (TWO) stage_block2<KMAX>(A, ldw, Yn, kq4, (i & 1) ? buf0 : buf1, lane);
+        else stage_block<KMAX>(A, ldw, Yn, kq4, (i & 1) ? buf0 : buf1, lane);
         adj_next = valid_u ? A[(int64_t)u * ldw + Yn.r * k + Yn.c] : 0u;
         col_next = lane < Yn.size ? A[(int64_t)(Yn.base + lane) * ldw + X.r * k + cu] : 0u;
       }
@@ -138,10 +146,17 @@ __device__ __forceinline__ void sweep_item(const GraphView &p, const WorkItem it
         prev_cv = cv;
       }
       pc.tests += __popc(adjw);
-      const uint32_t open = plane0_unsettled<KMAX>(Fu, P, sv, adjw, k);
+      uint32_t open;
+      if constexpr (TWO) {
+        spread_plane1<KMAX>(sv, Y.size, k, lane);
+        __syncwarp();
+        open = two_unsettled<KMAX>(Fu, F1, P, sv, adjw, k);
+      } else {
+        open = plane0_unsettled<KMAX>(Fu, P, sv, adjw, k);
+      }
       uint32_t del = 0;
       if (open)
-        del = recount_unsettled(rowu, sv, KMAX, A + (int64_t)Y.base * ldw, ldw, open, k, cu, cv, p.rounds, 0);
+        del = recount_unsettled(rowu, sv, kRow, A + (int64_t)Y.base * ldw, ldw, open, k, cu, cv, p.rounds, 0);
       const int wy = Y.r * k + cv;
       if (valid_u) An[(int64_t)u * ldw + wy] = adjw & ~del;
       pc.de += __popc(del);
