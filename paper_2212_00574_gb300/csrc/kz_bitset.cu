@@ -679,8 +679,6 @@ kz_status bitset_finish_load(kz_graph g, cudaStream_t s) {
     KZ_CUDA_TRY(cudaMemsetAsync(g->d_changed, 0xff, (size_t)std::max<int64_t>(g->n_units, 1), s));
     KZ_TRY(ensure_plan(g, g->form, s));
   }
-  KZ_TRY(graph_alloc(g, &g->A[0], (size_t)g->n * g->ldw, s));
-  KZ_TRY(graph_alloc(g, &g->A[1], (size_t)g->n * g->ldw, s));
   KZ_TRY(graph_alloc(g, &g->v_sweep, (size_t)std::max(g->n, 1), s));
   if (!g->st) {
     KZ_TRY(graph_alloc(g, &g->st, 1, s));
@@ -692,10 +690,11 @@ kz_status bitset_finish_load(kz_graph g, cudaStream_t s) {
 
 kz_status bitset_reset(kz_graph g, cudaStream_t s) {
   const size_t abytes = (size_t)g->n * g->ldw * 4;
-  if (abytes) {
+  if (abytes && !g->live_packed) {
     KZ_CUDA_TRY(cudaMemcpyAsync(g->A[0], g->A0, abytes, cudaMemcpyDeviceToDevice, s));
     KZ_CUDA_TRY(cudaMemcpyAsync(g->A[1], g->A0, abytes, cudaMemcpyDeviceToDevice, s));
   }
+  g->live_packed = false;  // later resets copy
   KZ_CUDA_TRY(cudaMemcpyAsync(g->V[0], g->V0, (size_t)g->ldw * 4, cudaMemcpyDeviceToDevice, s));
   KZ_CUDA_TRY(cudaMemcpyAsync(g->V[1], g->V0, (size_t)g->ldw * 4, cudaMemcpyDeviceToDevice, s));
   if (g->n) KZ_CUDA_TRY(cudaMemsetAsync(g->v_sweep, 0, sizeof(int32_t) * g->n, s));

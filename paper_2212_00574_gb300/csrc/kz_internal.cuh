@@ -89,6 +89,7 @@ struct kz_graph_s {
   // device buffers (owned)
   uint32_t *A0 = nullptr;     // pristine adjacency, n * ldw words
   uint32_t *A[2] = {nullptr, nullptr};
+  bool live_packed = false;   // the packer filled A[0] and A[1] too
   uint32_t *V0 = nullptr;     // pristine live words, ldw
   uint32_t *V[2] = {nullptr, nullptr};
   int32_t *v_sweep = nullptr;  // n (relabelled ids)

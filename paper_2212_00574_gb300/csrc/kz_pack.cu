@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "kz_internal.cuh"
+#include "kz_pack_tiles.cuh"
 #include "kz_rules.cuh"
 
 namespace kz {
@@ -182,101 +183,41 @@ __global__ void __launch_bounds__(kPackThreads) pack_dense_rows_kernel(PackArgs 
   if ((threadIdx.x & 31) == 0 && mine) atomicAdd(a.edge_count, mine);
 }
 
-// Tile form of the dense packer, first half, over caller rows [r0, r1): the
-// relabelling moves columns, so a CTA takes 32 caller rows i0 .. i0 + 31 at
-// a time and turns the bit permutation into a word gather between two warp
-// transposes.  (1) Column words: lane r reads 32 bytes of row i0 + r (every
-// sector used), and per 32 columns a transpose gives lane b the word of
-// column 32 q + b over the 32 rows, kept in shared memory (colw, one word
-// per caller column).  (2) Output: for word w = rr k + c of the relabelled
-// rows, lane b fetches the column word of caller column perm[y], y = coff[c]
-// + 32 rr + b, keeps only the rows r with i0 + r < perm[y] (the upper
-// triangle; symmetrize_kernel adds the other half), and a transpose gives
-// lane r word w of row inv[i0 + r].  Lane r collects kTileWords consecutive
-// words before one 32-byte store.  A set bit in an own-class word is an edge
-// inside one class: an illegal colouring.  colw takes 4 bytes per caller
-// column, so this form serves graphs up to kTileMaxN vertices; larger ones
-// take the row form.
-constexpr int kTileThreads = 512;
-constexpr int kTileWords = 8;
+// Tile form of the dense packer over caller rows [r0, r1), r0 a multiple of
+// 32 (kz_pack_tiles.cuh): symmetric rows in one pass, written to the pristine
+// copy and to both live buffers, for which the rows [0, r1) suffice.  One
+// column word per caller column takes 4 n bytes of shared memory, so this
+// form serves graphs up to kTileMaxN vertices; larger ones take the row form.
 constexpr int kTileMaxN = 48 * 1024;
 constexpr size_t kTileSmemBytes = 216 * 1024;
 
-__global__ void __launch_bounds__(kTileThreads) pack_dense_tiles_kernel(PackArgs a, const uint64_t *__restrict__ bits,
+__global__ void __launch_bounds__(kTileThreads) pack_dense_tiles_kernel(PackArgs a, uint32_t *__restrict__ A1,
+                                                                       uint32_t *__restrict__ A2,
+                                                                       const uint64_t *__restrict__ bits,
                                                                        int64_t row_words, int32_t n, int32_t R,
                                                                        const int32_t *__restrict__ perm, int64_t r0,
                                                                        int64_t r1) {
   extern __shared__ __align__(16) uint32_t colw[];  // 32 * ceil(n / 32) column words
-  const int nq = (n + 31) >> 5;
-  int32_t *scoff = reinterpret_cast<int32_t *>(colw + 32 * nq);  // k + 1
-  const int k = a.k, rk = R * k;
-  for (int c = threadIdx.x; c <= k; c += blockDim.x) scoff[c] = a.coff[c];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  int32_t *scoff = reinterpret_cast<int32_t *>(colw + (n + 31) / 32 * 32);  // k + 1
+  for (int c = threadIdx.x; c <= a.k; c += blockDim.x) scoff[c] = a.coff[c];
+  const int lane = threadIdx.x & 31;
   unsigned long long mine = 0;
+  bool bad = false;
   for (int64_t i0 = r0 + (int64_t)blockIdx.x * 32; i0 < r1; i0 += (int64_t)gridDim.x * 32) {
     const int rows = r1 - i0 < 32 ? (int)(r1 - i0) : 32;
     __syncthreads();  // the previous rows' column words are consumed (and scoff is written)
-    // (1) column words, kTileWords 32-bit words (256 columns) of a row per lane
-    const uint64_t *row = bits + (i0 + lane) * row_words;
-    for (int q0 = warp * kTileWords; q0 < nq; q0 += nwarps * kTileWords) {
-      uint32_t v[kTileWords];
-#pragma unroll
-      for (int u = 0; u < kTileWords; u += 2) {
-        const int64_t w64 = (q0 + u) >> 1;
-        const uint64_t x = (lane < rows && w64 < row_words) ? row[w64] : 0ull;
-        v[u] = (uint32_t)x;
-        v[u + 1] = (uint32_t)(x >> 32);
-      }
-#pragma unroll
-      for (int u = 0; u < kTileWords; u++) {
-        const uint32_t col = transpose32(v[u]);
-        if (q0 + u < nq) colw[32 * (q0 + u) + lane] = col;
-      }
-    }
+    tile_columns(colw, bits, row_words, n, i0, rows);
     __syncthreads();
-    const int64_t i = i0 + lane;  // this lane's row after the second transpose
-    const int32_t x = lane < rows ? a.inv[i] : 0;
-    const int own = lane < rows ? a.col[x] : -1;
-    // (2) the relabelled words, kTileWords per lane before a store
-    for (int w0 = warp * kTileWords; w0 < a.ldw; w0 += nwarps * kTileWords) {
-      uint32_t out[kTileWords];
-      int c = w0 % k, rr = w0 / k;  // class and round of word w0 + u
-#pragma unroll
-      for (int u = 0; u < kTileWords; u++) {
-        uint32_t col = 0u;
-        if (w0 + u < rk) {
-          const int32_t y = scoff[c] + 32 * rr + lane;
-          if (y < scoff[c + 1]) {
-            const int32_t j = perm[y];
-            const int64_t above = (int64_t)j - i0;  // rows r < above lie above the diagonal
-            const uint32_t keep = above >= 32 ? 0xffffffffu : above <= 0 ? 0u : ((1u << above) - 1u);
-            col = colw[j] & keep;
-          }
-        }
-        out[u] = transpose32(col);
-        if (out[u] && w0 + u < rk && c == own) {
-          atomicCAS(a.error, 0, (int32_t)KZ_ERR_ILLEGAL_COLOURING);
-          out[u] = 0u;
-        }
-        if (++c == k) {
-          c = 0;
-          ++rr;
-        }
-      }
-      if (lane < rows) {
-        uint32_t *dst = a.A + (int64_t)x * a.ldw + w0;
-        *reinterpret_cast<uint4 *>(dst) = make_uint4(out[0], out[1], out[2], out[3]);
-        if (w0 + kTileWords <= a.ldw) *reinterpret_cast<uint4 *>(dst + 4) = make_uint4(out[4], out[5], out[6], out[7]);
-        mine += __popc(out[0]) + __popc(out[1]) + __popc(out[2]) + __popc(out[3]);
-        if (w0 + kTileWords <= a.ldw) mine += __popc(out[4]) + __popc(out[5]) + __popc(out[6]) + __popc(out[7]);
-      }
-    }
+    const bool valid = lane < rows;
+    const int32_t x = valid ? a.inv[i0 + lane] : 0;
+    mine += tile_rows(colw, a.A, A1, A2, a.ldw, a.k, R, scoff, perm, x, valid ? a.col[x] : -1, valid, &bad);
   }
+  if (bad) atomicCAS(a.error, 0, (int32_t)KZ_ERR_ILLEGAL_COLOURING);
   for (int o = 16; o > 0; o >>= 1) mine += __shfl_down_sync(0xffffffffu, mine, o);
-  if ((threadIdx.x & 31) == 0 && mine) atomicAdd(a.edge_count, mine);
+  if (lane == 0 && mine) atomicAdd(a.edge_count, mine);
 }
 
-// Second half: every 32 x 32 tile of rows of block X (word position p of
+// Second half of the row form: every 32 x 32 tile of rows of block X (word position p of
 // the layout, p = r k + c: members 32 r .. 32 r + 31 of class c) at the word
 // of block Y becomes the OR of itself and the transpose of the tile of Y's
 // rows at X's word, and that tile the transpose of the result.  The word
@@ -598,10 +539,12 @@ kz_status bitset_vertex_alive(kz_graph g, uint8_t *host_alive, int64_t *n_live) 
 }
 
 // Shared set-up of the two packers: relabelling tables on the device and the
-// zeroed pristine adjacency.  Returns the temporaries to free after the sync.
-static kz_status pack_setup(kz_graph g, cudaStream_t s, PackArgs &a, std::vector<void *> &tmp) {
+// row buffers, the pristine one zeroed on request.  Returns the temporaries to free after the sync.
+static kz_status pack_setup(kz_graph g, cudaStream_t s, PackArgs &a, std::vector<void *> &tmp, bool zero) {
   KZ_TRY(graph_alloc(g, &g->A0, (size_t)g->n * g->ldw, s));
-  if (g->n > 0 && g->ldw > 0)
+  KZ_TRY(graph_alloc(g, &g->A[0], (size_t)g->n * g->ldw, s));
+  KZ_TRY(graph_alloc(g, &g->A[1], (size_t)g->n * g->ldw, s));
+  if (zero && g->n > 0 && g->ldw > 0)
     KZ_CUDA_TRY(cudaMemsetAsync(g->A0, 0, (size_t)g->n * g->ldw * 4, s));
   std::vector<int32_t> col_new((size_t)g->n);
   for (int c = 0; c < g->k; c++)
@@ -654,7 +597,7 @@ kz_status bitset_pack_edges(kz_graph g, const int32_t *d_edges, int64_t m, bool 
                             cudaStream_t s) {
   PackArgs a;
   std::vector<void *> tmp;
-  kz_status st = pack_setup(g, s, a, tmp);
+  kz_status st = pack_setup(g, s, a, tmp, true);
   if (st == KZ_OK && m > 0) {
     const int threads = 256;
     const int grid = (int)std::min<int64_t>((m + threads - 1) / threads, 64 * sm_count());
@@ -668,23 +611,22 @@ kz_status bitset_pack_edges(kz_graph g, const int32_t *d_edges, int64_t m, bool 
 kz_status bitset_pack_dense(kz_graph g, const uint64_t *h_bits, int64_t row_words, cudaStream_t s) {
   PackArgs a;
   std::vector<void *> tmp;
-  kz_status st = pack_setup(g, s, a, tmp);
+  // the tile form while one column word per caller column fits in shared
+  // memory (32 rows x n bits); it writes every word, the row form the upper
+  // triangle of zeroed rows, which a second kernel makes symmetric
+  const size_t row = (size_t)((g->n + 31) / 32) * 4, coff = (size_t)(g->k + 1) * 4;
+  const bool tiles = g->n <= kTileMaxN && 32 * row + coff <= kTileSmemBytes;
+  kz_status st = pack_setup(g, s, a, tmp, !tiles);
   const int64_t words = (int64_t)g->n * g->ldw;
   if (st == KZ_OK && words > 0) {
-    // the upper triangle row by row, then the transposed half tile by tile
-    const size_t row = (size_t)((g->n + 31) / 32) * 4, coff = (size_t)(g->k + 1) * 4;
     if (row + coff > kRowSmemBytes) st = KZ_ERR_UNSUPPORTED;  // beyond the bitset budget's reach
-    // the tile form while one column word per caller column fits in shared
-    // memory (32 rows x n bits)
-    const bool tiles = g->n <= kTileMaxN && 32 * row + coff <= kTileSmemBytes;
     const int rows = tiles ? 32 : 4 * row + coff <= kRowSmemBytes ? 4 : 2 * row + coff <= kRowSmemBytes ? 2 : 1;
     const int threads = tiles ? kTileThreads : kPackThreads;
     const size_t smem = rows * row + coff;
-    auto fn = tiles ? pack_dense_tiles_kernel
-                    : rows == 4 ? pack_dense_rows_kernel<4> : rows == 2 ? pack_dense_rows_kernel<2> : pack_dense_rows_kernel<1>;
+    auto row_fn = rows == 4 ? pack_dense_rows_kernel<4> : rows == 2 ? pack_dense_rows_kernel<2> : pack_dense_rows_kernel<1>;
+    const void *fn = tiles ? (const void *)pack_dense_tiles_kernel : (const void *)row_fn;
     int per_sm = 0;
-    if (st == KZ_OK)
-      st = cuda_status(cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (st == KZ_OK) st = cuda_status(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (st == KZ_OK) st = cuda_status(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem));
     const size_t bytes = (size_t)g->n * row_words * 8;
     uint64_t *d_bits = st == KZ_OK ? (uint64_t *)dev_alloc(bytes, s) : nullptr;
@@ -695,7 +637,7 @@ kz_status bitset_pack_dense(kz_graph g, const uint64_t *h_bits, int64_t row_word
     const int chunks = copy_chunks(bytes);
     cudaStream_t cs = chunks > 1 ? copy_stream() : s;
     if (st == KZ_OK && chunks > 1 && !cs) st = KZ_ERR_CUDA;
-    const int64_t per = ((int64_t)g->n + chunks - 1) / chunks;
+    const int64_t per = (((int64_t)g->n + chunks - 1) / chunks + 31) / 32 * 32;  // whole row groups
     std::vector<cudaEvent_t> ev;
     if (st == KZ_OK && cs != s) {
       ev.assign((size_t)chunks + 1, nullptr);
@@ -716,11 +658,15 @@ kz_status bitset_pack_dense(kz_graph g, const uint64_t *h_bits, int64_t row_word
       if (st != KZ_OK) break;
       const int64_t groups = (r1 - r0 + rows - 1) / rows;
       const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(groups, (int64_t)std::max(per_sm, 1) * sm_count()));
-      fn<<<grid, threads, smem, s>>>(a, d_bits, row_words, g->n, g->R, g->d_perm, r0, r1);
+      if (tiles)
+        pack_dense_tiles_kernel<<<grid, threads, smem, s>>>(a, g->A[0], g->A[1], d_bits, row_words, g->n, g->R,
+                                                            g->d_perm, r0, r1);
+      else
+        row_fn<<<grid, threads, smem, s>>>(a, d_bits, row_words, g->n, g->R, g->d_perm, r0, r1);
       st = cuda_status(cudaGetLastError());
     }
     if (st != KZ_OK && copied_any && cs != s) cudaStreamSynchronize(cs);  // no release under a running copy
-    if (st == KZ_OK) {
+    if (st == KZ_OK && !tiles) {
       const int64_t ng = ((int64_t)g->R * g->k + kSymGroup - 1) / kSymGroup;
       const int64_t pairs = ng * (ng + 1) / 2;
       const int sgrid = (int)std::max<int64_t>(1, std::min<int64_t>(pairs, 8 * sm_count()));
@@ -731,8 +677,12 @@ kz_status bitset_pack_dense(kz_graph g, const uint64_t *h_bits, int64_t row_word
       if (e) cudaEventDestroy(e);
     if (d_bits) dev_free(d_bits, bytes, s);
   }
-  kz_status st2 = st == KZ_OK ? pack_finish(g, s, a, tmp) : KZ_OK;
-  return st != KZ_OK ? st : st2;
+  if (st == KZ_OK) st = pack_finish(g, s, a, tmp);
+  if (st == KZ_OK && tiles) {
+    g->m /= 2;  // the tile form counts both halves
+    g->live_packed = true;
+  }
+  return st;
 }
 
 }  // namespace kz
