@@ -62,30 +62,101 @@ using namespace kz::mlp;
 // MLP kernels (tensor cores: warp-level bf16 MMAs, see kz_mlp.cuh)
 // ---------------------------------------------------------------------------
 
-constexpr int kFwdWarps = 8;
-
 // Logits of B feature rows X (fp32 [B][16]), 32 rows per warp step.
-__global__ void __launch_bounds__(32 * kFwdWarps) mlp_forward_kernel(const __nv_bfloat16 *__restrict__ w16,
-                                                                      const float *__restrict__ X, int64_t B,
-                                                                      float *__restrict__ logits) {
-  __shared__ SmemNet net;
-  __shared__ __align__(16) __nv_bfloat16 sx[kFwdWarps][kTileRows * kXLd];
-  load_net(net, w16);
-  uint32_t w1f[8][2];
-  load_w1_frags(w1f, w16);
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t stride = (int64_t)gridDim.x * kFwdWarps * kTileRows;
-  for (int64_t base = ((int64_t)blockIdx.x * kFwdWarps + warp) * kTileRows; base < B; base += stride) {
-    const int64_t q = base + lane;
-    float f[F];
+//
+// What bounds it: the rate of mma.sync (80 MMAs per 32 rows).  W1 and W2 stay
+// in registers as B fragments (80 registers a thread) and the feature rows go
+// straight from global memory into A fragments (the four lanes of a quad read
+// 32 bytes of a row), one step ahead; only the bias and output vectors come
+// from shared memory.  With W2 and the features in shared memory that pipe
+// was 88% busy and the tensor pipe 35%.  1,000,003 rows: 53 us before,
+// 31 us now (4,000,000: 198 and 112 us, 370 TFLOP/s; the tensor pipe is 63% busy).
+// (The MMAs, their order and every rounding are those of tile_logits, so the
+// logits are the same bits.)
+constexpr int kFwdWarps = 4;
+
+__device__ __forceinline__ void load_rows(float2 (&f)[2][4], const float *__restrict__ X, int64_t base, int64_t B,
+                                          int g, int t) {
 #pragma unroll
-    for (int i = 0; i < F; i++) f[i] = q < B ? X[q * F + i] : 0.f;
-    store_row(sx[warp] + lane * kXLd, f);
-    __syncwarp();
-    const float l = tile_logits(net, w1f, sx[warp]);
-    if (q < B) logits[q] = l;
-    __syncwarp();
+  for (int mt = 0; mt < 2; mt++)
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+      const int64_t q = base + 16 * mt + 8 * h + g;
+      const float2 *row = reinterpret_cast<const float2 *>(X + q * F);
+      f[mt][h] = q < B ? __ldg(row + t) : make_float2(0.f, 0.f);
+      f[mt][2 + h] = q < B ? __ldg(row + t + 4) : make_float2(0.f, 0.f);
+    }
+}
+
+__global__ void __launch_bounds__(32 * kFwdWarps, 2) mlp_forward_kernel(const __nv_bfloat16 *__restrict__ w16,
+                                                                        const float *__restrict__ X, int64_t B,
+                                                                        float *__restrict__ logits) {
+  __shared__ float2 sb1[H / 2], sb2[H / 2], sw3[H / 2];
+  for (int j = threadIdx.x; j < H / 2; j += blockDim.x) {
+    sb1[j] = make_float2(__bfloat162float(w16[ob1 + 2 * j]), __bfloat162float(w16[ob1 + 2 * j + 1]));
+    sb2[j] = make_float2(__bfloat162float(w16[ob2 + 2 * j]), __bfloat162float(w16[ob2 + 2 * j + 1]));
+    sw3[j] = make_float2(__bfloat162float(w16[ow3 + 2 * j]), __bfloat162float(w16[ow3 + 2 * j + 1]));
+  }
+  const float b3 = __bfloat162float(w16[ob3]);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  uint32_t w1f[8][2], w2f[8][4][2];
+  load_w1_frags(w1f, w16);
+#pragma unroll
+  for (int nt = 0; nt < 8; nt++)
+#pragma unroll
+    for (int s = 0; s < 4; s++) {
+      const __nv_bfloat16 *wr = w16 + oW2 + (8 * nt + g) * H + 16 * s + 2 * t;
+      w2f[nt][s][0] = ld_u32(wr);
+      w2f[nt][s][1] = ld_u32(wr + 8);
+    }
+  __syncthreads();
+  const int64_t stride = (int64_t)gridDim.x * kFwdWarps * kTileRows;
+  int64_t base = ((int64_t)blockIdx.x * kFwdWarps + warp) * kTileRows;
+  float2 f[2][4];
+  if (base < B) load_rows(f, X, base, B, g, t);
+  for (; base < B; base += stride) {
+    uint32_t a[2][4];
+#pragma unroll
+    for (int mt = 0; mt < 2; mt++)
+#pragma unroll
+      for (int i = 0; i < 4; i++) a[mt][i] = pack_bf16x2(f[mt][i].x, f[mt][i].y);
+    if (base + stride < B) load_rows(f, X, base + stride, B, g, t);
+#pragma unroll
+    for (int mt = 0; mt < 2; mt++) {
+      uint32_t a2[4][4];
+#pragma unroll
+      for (int s = 0; s < 4; s++) {
+        float c[2][4];
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+          const float2 b1 = sb1[4 * (2 * s + h) + t];
+          c[h][0] = c[h][2] = b1.x;
+          c[h][1] = c[h][3] = b1.y;
+          mma_bf16_16816(c[h], a[mt], w1f[2 * s + h][0], w1f[2 * s + h][1]);
+        }
+        a2[s][0] = pack_bf16x2(fmaxf(c[0][0], 0.f), fmaxf(c[0][1], 0.f));
+        a2[s][1] = pack_bf16x2(fmaxf(c[0][2], 0.f), fmaxf(c[0][3], 0.f));
+        a2[s][2] = pack_bf16x2(fmaxf(c[1][0], 0.f), fmaxf(c[1][1], 0.f));
+        a2[s][3] = pack_bf16x2(fmaxf(c[1][2], 0.f), fmaxf(c[1][3], 0.f));
+      }
+      float out[2] = {0.f, 0.f};
+#pragma unroll
+      for (int nt = 0; nt < 8; nt++) {
+        const float2 b2 = sb2[4 * nt + t], w3 = sw3[4 * nt + t];
+        float c[4] = {b2.x, b2.y, b2.x, b2.y};
+#pragma unroll
+        for (int s = 0; s < 4; s++) mma_bf16_16816(c, a2[s], w2f[nt][s][0], w2f[nt][s][1]);
+        out[0] = fmaf(w3.x, fmaxf(c[0], 0.f), fmaf(w3.y, fmaxf(c[1], 0.f), out[0]));
+        out[1] = fmaf(w3.x, fmaxf(c[2], 0.f), fmaf(w3.y, fmaxf(c[3], 0.f), out[1]));
+      }
+#pragma unroll
+      for (int h = 0; h < 2; h++) {
+        out[h] += __shfl_xor_sync(0xffffffffu, out[h], 1);
+        out[h] += __shfl_xor_sync(0xffffffffu, out[h], 2);
+        const int64_t q = base + 16 * mt + 8 * h + g;
+        if (t == 0 && q < B) logits[q] = out[h] + b3;
+      }
+    }
   }
 }
 
@@ -96,6 +167,9 @@ __global__ void __launch_bounds__(32 * kFwdWarps) mlp_forward_kernel(const __nv_
 // shared memory, transposed to [feature or hidden unit][sample]; then every
 // warp forms 16 rows of dW2 = dz2^T h1 and dW1 = dz1^T x over the chunk's
 // samples (K = samples), accumulated in registers across the CTA's chunks.
+// A training step (4096 rows) is one chunk a CTA, so it is bound by latency:
+// W2 arrives in 16-byte loads and the sums leave as pair reductions (12.3 us
+// to 10.8 us; 65,536 rows, with the step's other launches: 53 to 47 us).
 constexpr int kGradWarps = 4;
 constexpr int kChunk = 16 * kGradWarps;
 constexpr int kSLd = kChunk + 8;  // row stride of the [unit][sample] tiles
@@ -124,6 +198,24 @@ __device__ __forceinline__ float column_sum(float v) {
   return v + __shfl_xor_sync(0xffffffffu, v, 16);
 }
 
+// Two neighbouring sums into the global gradient: one vector reduction when
+// the caller's buffer is 8-byte aligned.
+__device__ __forceinline__ void add_pair(float *p, float a, float b, bool pair) {
+  if (pair) {
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b) : "memory");
+  } else {
+    atomicAdd(p, a);
+    atomicAdd(p + 1, b);
+  }
+}
+
+// The gradient and loss buffers emptied by one launch.
+__global__ void zero_grad_kernel(float *__restrict__ grad, float *__restrict__ loss) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < P) grad[i] = 0.f;
+  if (i == P) *loss = 0.f;
+}
+
 __global__ void __launch_bounds__(32 * kGradWarps) mlp_grad_kernel(const __nv_bfloat16 *__restrict__ w16,
                                                                     const float *__restrict__ X,
                                                                     const float *__restrict__ y, int64_t B,
@@ -133,7 +225,15 @@ __global__ void __launch_bounds__(32 * kGradWarps) mlp_grad_kernel(const __nv_bf
   GradSmem &S = *reinterpret_cast<GradSmem *>(smraw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   load_net(S.net, w16);
-  for (int e = tid; e < H * H; e += blockDim.x) S.W2T[(e % H) * kWLd + e / H] = w16[oW2 + e];
+  // W2 transposed, from 16-byte loads
+  for (int e = tid; e < H * H / 8; e += blockDim.x) {
+    const int j = e / (H / 8), i = 8 * (e % (H / 8));
+    const uint4 w = ld_w16x8(w16 + oW2 + 8 * e);
+    const uint32_t q[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int u = 0; u < 8; u++)
+      S.W2T[(i + u) * kWLd + j] = __ushort_as_bfloat16((unsigned short)(q[u >> 1] >> (16 * (u & 1))));
+  }
   for (int j = tid; j < H; j += blockDim.x) S.gb1[j] = S.gb2[j] = S.gw3[j] = 0.f;
   if (tid == 0) S.gb3 = S.loss = 0.f;
   uint32_t w1f[8][2];
@@ -307,22 +407,19 @@ __global__ void __launch_bounds__(32 * kGradWarps) mlp_grad_kernel(const __nv_bf
   }
   // this CTA's sums into the global gradient
   {
+    const bool pair = (reinterpret_cast<uintptr_t>(grad) & 7u) == 0;  // (oW1, oW2 and i are even)
     const int j0 = 16 * warp + g;
 #pragma unroll
     for (int nt = 0; nt < 8; nt++) {
       const int i = 8 * nt + 2 * t;
-      atomicAdd(&grad[oW2 + j0 * H + i], accW2[nt][0]);
-      atomicAdd(&grad[oW2 + j0 * H + i + 1], accW2[nt][1]);
-      atomicAdd(&grad[oW2 + (j0 + 8) * H + i], accW2[nt][2]);
-      atomicAdd(&grad[oW2 + (j0 + 8) * H + i + 1], accW2[nt][3]);
+      add_pair(&grad[oW2 + j0 * H + i], accW2[nt][0], accW2[nt][1], pair);
+      add_pair(&grad[oW2 + (j0 + 8) * H + i], accW2[nt][2], accW2[nt][3], pair);
     }
 #pragma unroll
     for (int nt = 0; nt < 2; nt++) {
       const int i = 8 * nt + 2 * t;
-      atomicAdd(&grad[oW1 + j0 * F + i], accW1[nt][0]);
-      atomicAdd(&grad[oW1 + j0 * F + i + 1], accW1[nt][1]);
-      atomicAdd(&grad[oW1 + (j0 + 8) * F + i], accW1[nt][2]);
-      atomicAdd(&grad[oW1 + (j0 + 8) * F + i + 1], accW1[nt][3]);
+      add_pair(&grad[oW1 + j0 * F + i], accW1[nt][0], accW1[nt][1], pair);
+      add_pair(&grad[oW1 + (j0 + 8) * F + i], accW1[nt][2], accW1[nt][3], pair);
     }
   }
   __syncthreads();
@@ -1651,8 +1748,7 @@ kz_status kz_mlp_grad(kz_model m, const float *X, const float *y, int64_t B, flo
       configured[dev] = true;
     }
   }
-  KZ_CUDA_TRY(cudaMemsetAsync(grad, 0, P * 4, s));
-  KZ_CUDA_TRY(cudaMemsetAsync(loss, 0, 4, s));
+  zero_grad_kernel<<<(P + 256) / 256, 256, 0, s>>>(grad, loss);
   const int64_t blocks = std::min<int64_t>((B + kChunk - 1) / kChunk, 2 * sms_now());
   mlp_grad_kernel<<<(unsigned)blocks, 32 * kGradWarps, smem, s>>>(m->w16, X, y, B, grad, loss);
   return cuda_status(cudaGetLastError());
@@ -1663,7 +1759,7 @@ kz_status kz_mlp_adam(kz_model m, const float *grad, float lr, void *stream) {
   m->t += 1;
   const float bc1 = 1.f - std::pow(0.9f, (float)m->t);
   const float bc2 = 1.f - std::pow(0.999f, (float)m->t);
-  adam_kernel<<<8, 256, 0, (cudaStream_t)stream>>>(m->w32, m->w16, m->m, m->v, grad, lr, bc1, bc2);
+  adam_kernel<<<(P + 255) / 256, 256, 0, (cudaStream_t)stream>>>(m->w32, m->w16, m->m, m->v, grad, lr, bc1, bc2);
   return cuda_status(cudaGetLastError());
 }
 

@@ -61,17 +61,23 @@ __device__ __forceinline__ uint32_t ld_u32(const __nv_bfloat16 *p) {
   return *reinterpret_cast<const uint32_t *>(p);
 }
 
+// Eight bf16 weights from an address of 16-byte alignment.
+__device__ __forceinline__ uint4 ld_w16x8(const __nv_bfloat16 *p) { return __ldg(reinterpret_cast<const uint4 *>(p)); }
+
 // The network's parameters as one CTA holds them: W2 in shared memory in its
 // [j][i] layout (padded rows), the small vectors widened to fp32.
 struct SmemNet {
-  __nv_bfloat16 W2[H * kWLd];
+  alignas(16) __nv_bfloat16 W2[H * kWLd];
   float b1[H], b2[H], w3[H];
   float b3;
 };
 
 // Cooperative load of the bf16 parameters into shared memory (whole block).
 __device__ __forceinline__ void load_net(SmemNet &s, const __nv_bfloat16 *__restrict__ w16) {
-  for (int e = threadIdx.x; e < H * H; e += blockDim.x) s.W2[(e / H) * kWLd + e % H] = w16[oW2 + e];
+  // (w16 is the model's own allocation and oW2 a multiple of 8; rows of W2
+  // are 144 bytes apart)
+  for (int e = threadIdx.x; e < H * H / 8; e += blockDim.x)
+    *reinterpret_cast<uint4 *>(s.W2 + (e / (H / 8)) * kWLd + 8 * (e % (H / 8))) = ld_w16x8(w16 + oW2 + 8 * e);
   for (int j = threadIdx.x; j < H; j += blockDim.x) {
     s.b1[j] = __bfloat162float(w16[ob1 + j]);
     s.b2[j] = __bfloat162float(w16[ob2 + j]);
