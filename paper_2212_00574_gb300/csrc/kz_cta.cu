@@ -19,6 +19,7 @@
 #include "kz_internal.cuh"
 #include "kz_pack_tiles.cuh"
 #include "kz_rules.cuh"
+#include "kz_small.cuh"
 #include "kz_sweep.cuh"
 
 namespace kz {
@@ -457,45 +458,6 @@ kz_status cta_kernelize_one(kz_graph g, const kz_options &opt, cudaStream_t s) {
 // the smallest graphs), reading its descriptor from that array.
 // ---------------------------------------------------------------------------
 
-namespace kz {
-namespace noalloc {
-
-constexpr int kMaxN = KZ_NOALLOC_MAX_N;
-constexpr int kMaxWords = KZ_NOALLOC_MAX_WORDS;  // words per adjacency buffer
-constexpr int kMaxLdw = 4096;                    // words per row
-constexpr int kMaxBlocks = 256;
-
-struct Header {
-  CtaGraph desc;
-  int32_t status;   // found by the set-up
-  int32_t illegal;  // KZ_ERR_ILLEGAL_COLOURING, found by the packer
-  int32_t R, pad;
-  int64_t cross;            // pairs of vertices in different classes
-  unsigned long long bits;  // set bits of the packed rows: twice the edges
-  int32_t coff[65];
-  int32_t boff[65];
-  int32_t rounds[64];
-  int32_t pair_off[kMaxBlocks + 1];
-  int32_t unit_off[kMaxBlocks + 1];  // prefix of the grid kernel's units: block pairs, one for a block without any
-  BlockDesc blocks[kMaxBlocks];
-};
-
-struct Scratch {
-  alignas(256) Header h;
-  alignas(256) DevState st;
-  alignas(256) uint32_t A0[kMaxWords];
-  alignas(256) uint32_t A1[kMaxWords];
-  alignas(256) uint32_t V0[kMaxLdw];
-  alignas(256) uint32_t V1[kMaxLdw];
-  alignas(256) int32_t perm[kMaxN];
-  alignas(256) int32_t inv[kMaxN];
-  alignas(256) int32_t pos[kMaxN];  // caller vertex -> (word << 5) | bit of its relabelled vertex inside any row
-  alignas(256) int32_t v_sweep[kMaxN];
-};
-
-}  // namespace noalloc
-}  // namespace kz
-
 // The scratch of kz_kernelize_dense_noalloc (about 9 MiB per device).
 static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(kz::noalloc::Scratch)];
 
@@ -797,6 +759,31 @@ static GridFn pick_grid(int k, int &kmax) {
 
 constexpr size_t grid_smem(int kmax) { return (size_t)kGridWarps * 2 * 32 * 2 * kmax * 4; }
 
+static kz_status configure_grid() {
+  for (int kk = 8; kk <= 32; kk += 8) {
+    int km = 0, per_sm = 0;
+    const GridFn fn = pick_grid(kk, km);
+    KZ_CUDA_TRY(cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)grid_smem(km)));
+    KZ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)fn, kGridWarps * 32,
+                                                              grid_smem(km)));
+    if (per_sm < 1) return KZ_ERR_UNSUPPORTED;
+  }
+  return KZ_OK;
+}
+
+// One CTA per SM at most (all resident, as the grid barrier needs), and no
+// more warps than the block pairs the classes can make.
+static kz_status launch_grid(Scratch *sp, int32_t n, int32_t k, int64_t max_sweeps, int sms, cudaStream_t s) {
+  int km = 0;
+  const GridFn fn = pick_grid(k, km);
+  const int64_t blocks = n / 32 + k, pairs = blocks * blocks / 2;
+  const int ctas = (int)std::max<int64_t>(1, std::min<int64_t>(std::max(sms, 1), (pairs + kGridWarps - 1) / kGridWarps));
+  void *args[] = {&sp, &max_sweeps};
+  KZ_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)fn, dim3(ctas), dim3(kGridWarps * 32), args, grid_smem(km), s));
+  return KZ_OK;
+}
+
 // Vertices up to which one CTA runs the fixpoint from shared memory: below
 // it a pass is shorter than a grid barrier (n = 100: 9.7 us a pass on one CTA,
 // n = 200: 8.1 us on the grid).
@@ -860,6 +847,11 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_kernel(Scratch *s, int3
 }
 
 }  // namespace noalloc
+
+void small_setup(noalloc::Scratch *s, int32_t n, int32_t k, const int32_t *colour, cudaStream_t stream) {
+  noalloc::setup_kernel<<<1, 1024, 0, stream>>>(s, n, k, colour);
+}
+
 }  // namespace kz
 
 namespace {
@@ -910,32 +902,16 @@ extern "C" kz_status kz_kernelize_dense_noalloc(int32_t n, int32_t k, const int3
     if (!configured[dev]) {
       KZ_CUDA_TRY(cudaFuncSetAttribute((const void *)fixpoint_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes));
-      // every width is set up (and loaded) now, so that no later call does
-      for (int kk = 8; kk <= 32; kk += 8) {
-        int km = 0, per_sm = 0;
-        const GridFn fn = pick_grid(kk, km);
-        KZ_CUDA_TRY(cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)grid_smem(km)));
-        KZ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)fn, kGridWarps * 32,
-                                                                  grid_smem(km)));
-        if (per_sm < 1) return KZ_ERR_UNSUPPORTED;
-      }
+      KZ_TRY(configure_grid());  // every width is set up (and loaded) now, so that no later call does
       configured[dev] = true;
     }
   }
-  setup_kernel<<<1, 1024, 0, s>>>(sp, n, k, colour);
+  kz::small_setup(sp, n, k, colour, s);
   if (n > 0) pack_kernel<<<(n + 31) / 32, kz::kTileThreads, (size_t)(n + 31) / 32 * 128, s>>>(sp, adj_bits, row_words, colour);
   if (n <= kOneCtaMaxN) {
     fixpoint_kernel<<<1, kz::kCtaThreads, smem_bytes, s>>>(sp, max_sweeps, smem_bytes / 4);
   } else {
-    // one CTA per SM at most (all resident, as the grid barrier needs), and no
-    // more warps than the block pairs the classes can make
-    int km = 0;
-    const GridFn fn = pick_grid(k, km);
-    const int64_t blocks = n / 32 + k, pairs = blocks * blocks / 2;
-    const int ctas = (int)std::min<int64_t>(std::max(sms, 1), (pairs + kGridWarps - 1) / kGridWarps);
-    void *args[] = {&sp, &max_sweeps};
-    KZ_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)fn, dim3(ctas), dim3(kGridWarps * 32), args, grid_smem(km), s));
+    KZ_TRY(launch_grid(sp, n, k, max_sweeps, sms, s));
   }
   unpack_kernel<<<std::max(1, std::min(n, 16 * std::max(sms, 1))), kUnpackThreads, 0, s>>>(sp, n, adj_out, row_words,
                                                                                           vertex_alive, counts);

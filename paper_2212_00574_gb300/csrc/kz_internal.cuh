@@ -127,19 +127,23 @@ struct kz_graph_s {
   // CSR path (caller ids)
   int64_t *sp_row0 = nullptr;  // n + 1, all edges
   int32_t *sp_adj0 = nullptr, *sp_eid0 = nullptr;
-  int64_t *sp_row[2] = {nullptr, nullptr};  // compacted live rows (ping-pong)
-  int32_t *sp_adj[2] = {nullptr, nullptr};
-  int32_t *sp_eid[2] = {nullptr, nullptr};
-  uint8_t *sp_elive[2] = {nullptr, nullptr};
-  uint8_t *sp_vlive[2] = {nullptr, nullptr};
-  int32_t sp_cur = 0;
-  int64_t *sp_orow = nullptr;  // oriented live CSR
-  int32_t *sp_oadj = nullptr, *sp_oeid = nullptr, *sp_osrc = nullptr;
+  int32_t *sp_adj = nullptr, *sp_eid = nullptr, *sp_len = nullptr;    // working rows: row u at sp_row0[u]
+  int32_t *sp_oadj = nullptr, *sp_oeid = nullptr, *sp_olen = nullptr; // oriented rows, at the same starts
+  uint8_t *sp_elive = nullptr, *sp_vlive = nullptr, *sp_vfail = nullptr;
+  int2 *sp_vinfo = nullptr;                  // rank, colour, fails in the running pass
+  int32_t *sp_list[2] = {nullptr, nullptr};  // live vertices of a pass and of the next
+  int2 *sp_items = nullptr;
+  int32_t *sp_big[2] = {nullptr, nullptr};
+  unsigned int *sp_ctr = nullptr;            // the lists' lengths, items, long-row edges
+  long long *sp_report = nullptr;
+  bool sp_from_input = true, sp_all_live = true;  // rows still the input's; no edge dead
+  bool sp_use_list = false;                  // of the running kernelize: the vertex list is built,
+  int sp_in = 0;                             // which list holds it,
+  int64_t sp_sweeps = 0, sp_tried = 0;       // sweeps so far, vertices of the last try of the bitset remnant
+  void *sp_small = nullptr;                  // remnant scratch (kz_small.cuh), on first use
   int32_t *sp_eu = nullptr, *sp_ev = nullptr;  // canonical sorted edges
   int32_t *sp_col = nullptr, *sp_rank = nullptr;
   unsigned long long *sp_mask = nullptr;
-  int32_t *sp_cnt_live = nullptr, *sp_cnt_or = nullptr;
-  int64_t *sp_sums = nullptr, *sp_totals = nullptr;
   int32_t *sp_v_sweep = nullptr;
 
   // learned schedule: attached model, threshold, per-graph scratch
@@ -260,8 +264,21 @@ kz_status sparse_kernelize(kz_graph g, const kz_options &opt, cudaStream_t s);
 kz_status sparse_fetch(kz_graph g, uint8_t *vertex_alive, int32_t *edges_out, int64_t cap, int64_t *m_live);
 kz_status sparse_vertex_alive(kz_graph g, uint8_t *host_alive, int64_t *n_live);
 kz_status sparse_v_sweep(kz_graph g, int32_t *host);
-// Oriented CSR of the live edges of the current CSR state.
+// What a pass of the CSR path left.
+struct SparseReport {
+  bool cont;               // the pass was applied and another follows
+  int64_t vertices;        // vertices on the next pass's list
+  int64_t live_before, live;  // live edges before and after
+};
+// One run's start, its passes one by one, and its end on bitset rows when the
+// live vertices fit (*done).
+kz_status sparse_begin(kz_graph g, int64_t max_sweeps, cudaStream_t s);
+kz_status sparse_one_pass(kz_graph g, int64_t max_sweeps, cudaStream_t s, SparseReport *out);
+kz_status sparse_finish_small(kz_graph g, int64_t max_sweeps, const SparseReport &r, cudaStream_t s, bool *done);
+// Working and oriented rows of the live edges; their triangles into per-class
+// edge counts (support schedule).
 kz_status sparse_orient_live(kz_graph g, cudaStream_t s);
+kz_status sparse_count_triangles(kz_graph g, uint32_t *cnt_e, cudaStream_t s);
 // The CSR path with incremental per-class support counts (kz_support.cu).
 kz_status sparse_kernelize_support(kz_graph g, const kz_options &opt, cudaStream_t s);
 void support_release(kz_graph g);

@@ -12,7 +12,9 @@
 // of the classes c != col v has count zero -- the rules of the thesis
 // restated with counts (a class is covered iff its count is positive).
 //
-// Sweep t:
+// The heavy sweeps at a run's start (more than a quarter of the live edges
+// deleted) are plain passes, and a remnant small enough for bitset rows ends
+// there; otherwise the counts are built and from then on, sweep t:
 //   1. rule: every dirty element (its counts changed in the last update; all
 //      live elements after a recount) is tested on the counts of S_t; the
 //      failing edges are listed;
@@ -20,8 +22,8 @@
 //      that loses an edge is visited once, from its deleted edge of smallest
 //      id, and each surviving edge of it loses that witness; each deleted
 //      edge decrements its endpoints' vertex counts.  The rows walked are
-//      the live rows compacted at the last recount (their dead entries are
-//      skipped).  After a sweep that deletes more than a quarter of the live
+//      the working rows of the last recount (their dead entries are skipped).
+//      After a sweep that deletes more than a quarter of the live
 //      edges the counts are recounted from scratch on the compacted live
 //      graph instead;
 //   3. apply: the live flags drop the failing elements.
@@ -94,40 +96,6 @@ __device__ __forceinline__ int64_t lower_bound_sorted(const int32_t *__restrict_
     else hi = mid;
   }
   return lo;
-}
-
-// Edge counts of the live graph: one warp per oriented live edge u -> v;
-// every live triangle is found once and adds its third vertex's class to
-// each of its three edges.
-__global__ void support_triangle_kernel(const int32_t *__restrict__ col, const int64_t *__restrict__ orow,
-                                        const int32_t *__restrict__ oadj, const int32_t *__restrict__ oeid,
-                                        const int32_t *__restrict__ osrc, const int64_t *__restrict__ n_or, int32_t k,
-                                        uint32_t *__restrict__ cnt_e) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = *n_or;
-  for (int64_t q = warp0; q < total; q += warps) {
-    const int32_t u = osrc[q], v = oadj[q], euv = oeid[q];
-    const int64_t ub = orow[u], ue = orow[u + 1];
-    const int64_t vb = orow[v], ve = orow[v + 1];
-    const bool walk_u = (ue - ub) <= (ve - vb);
-    const int64_t wb = walk_u ? ub : vb, we = walk_u ? ue : ve;
-    const int64_t sb = walk_u ? vb : ub, se = walk_u ? ve : ue;
-    const int32_t cu = col[u], cv = col[v];
-    for (int64_t i = wb + lane; i < we; i += 32) {
-      const int32_t w = oadj[i];
-      const int64_t j = lower_bound_sorted(oadj, sb, se, w);
-      if (j < se && oadj[j] == w) {
-        const int32_t e_walk = oeid[i], e_srch = oeid[j];
-        const int32_t euw = walk_u ? e_walk : e_srch;
-        const int32_t evw = walk_u ? e_srch : e_walk;
-        atomicAdd(&cnt_e[(int64_t)euv * k + col[w]], 1u);
-        atomicAdd(&cnt_e[(int64_t)euw * k + cv], 1u);
-        atomicAdd(&cnt_e[(int64_t)evw * k + cu], 1u);
-      }
-    }
-  }
 }
 
 // Step 1: the dirty live elements tested on the counts of the snapshot.
@@ -208,7 +176,7 @@ __global__ void support_rule_kernel(const int32_t *__restrict__ eu, const int32_
 // a smaller id; each surviving edge of the triangle loses the witness across.
 __global__ void support_update_kernel(const int32_t *__restrict__ eu, const int32_t *__restrict__ ev,
                                       const int32_t *__restrict__ col, const int64_t *__restrict__ row,
-                                      const int32_t *__restrict__ adj, const int32_t *__restrict__ eid,
+                                      const int32_t *__restrict__ len, const int32_t *__restrict__ adj, const int32_t *__restrict__ eid,
                                       const uint8_t *__restrict__ elive, const uint8_t *__restrict__ edel,
                                       const int32_t *__restrict__ dlist, const unsigned int *__restrict__ dcount,
                                       int32_t k, uint32_t *__restrict__ cnt_e, uint32_t *__restrict__ cnt_v,
@@ -227,8 +195,8 @@ __global__ void support_update_kernel(const int32_t *__restrict__ eu, const int3
       vdirty[u] = 1;
       vdirty[v] = 1;
     }
-    const int64_t ub = row[u], ue = row[u + 1];
-    const int64_t vb = row[v], ve = row[v + 1];
+    const int64_t ub = row[u], ue = ub + len[u];
+    const int64_t vb = row[v], ve = vb + len[v];
     const bool walk_u = (ue - ub) <= (ve - vb);
     const int64_t wb = walk_u ? ub : vb, we = walk_u ? ue : ve;
     const int64_t sb = walk_u ? vb : ub, se = walk_u ? ve : ue;
@@ -274,17 +242,6 @@ __global__ void support_finish_kernel(DevState *st) {
   st->pass_dv = st->pass_de = st->pass_tests = 0;
 }
 
-__global__ void support_begin_kernel(DevState *st, int64_t max_sweeps, int64_t passes0) {
-  st->status = KZ_OK;
-  st->cont = 1;
-  st->sweeps = 0;
-  st->passes = passes0;
-  st->tests = 0;
-  st->max_sweeps = max_sweeps;
-  st->pass_dv = st->pass_de = st->pass_tests = 0;
-  st->ticket = 0;
-}
-
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
@@ -321,33 +278,26 @@ void support_release(kz_graph g) {
   g->support_bufs = nullptr;
 }
 
-// Counts from scratch for the current live state: the plain path's
-// compaction (the live rows, compacted, land in the other row buffer; the
-// oriented CSR of the live edges beside them), then the per-class vertex and
-// edge counts; every live element is marked dirty.  Returns the live edges.
-static kz_status support_recount(kz_graph g, SupportBufs *b, cudaStream_t s, int64_t *live_edges) {
+// Counts from scratch for the current live state: the working and oriented
+// rows of the live edges, then the per-class vertex and edge counts; every
+// live element is marked dirty.
+static kz_status support_recount(kz_graph g, SupportBufs *b, cudaStream_t s) {
   const int grid = 8 * sms_of_device(), threads = 256;
   const int64_t n = g->n, m = g->m;
   const int k = g->k;
-  const int c = g->sp_cur;
-  uint8_t *elive = g->sp_elive[c], *vlive = g->sp_vlive[c];
   KZ_CUDA_TRY(cudaMemsetAsync(b->cnt_e, 0, sizeof(uint32_t) * (size_t)std::max<int64_t>(m, 1) * k, s));
   KZ_CUDA_TRY(cudaMemsetAsync(b->cnt_v, 0, sizeof(uint32_t) * (size_t)n * k, s));
-  support_init_kernel<<<grid, threads, 0, s>>>(g->sp_eu, g->sp_ev, g->sp_col, elive, vlive, m, (int32_t)n, k,
-                                               b->cnt_v, b->edirty, b->vdirty);
-  KZ_TRY(sparse_orient_live(g, s));
-  support_triangle_kernel<<<grid, threads, 0, s>>>(g->sp_col, g->sp_orow, g->sp_oadj, g->sp_oeid, g->sp_osrc,
-                                                   g->sp_totals + 1, k, b->cnt_e);
+  support_init_kernel<<<grid, threads, 0, s>>>(g->sp_eu, g->sp_ev, g->sp_col, g->sp_elive, g->sp_vlive, m, (int32_t)n,
+                                               k, b->cnt_v, b->edirty, b->vdirty);
   KZ_CUDA_TRY(cudaGetLastError());
-  KZ_CUDA_TRY(cudaMemcpyAsync(live_edges, g->sp_totals + 1, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  KZ_CUDA_TRY(cudaStreamSynchronize(s));
-  return KZ_OK;
+  KZ_TRY(sparse_orient_live(g, s));
+  return sparse_count_triangles(g, b->cnt_e, s);
 }
 
 // A sweep that deletes more than this share of the live edges is followed by
-// a recount from scratch instead of the incremental update: the update
-// visits every triangle a deleted edge closes (atomics on counts shared by
-// hub edges), while a recount enumerates the much smaller surviving graph.
+// another from scratch: as a plain pass of the CSR path while the run has no
+// counts yet, by a recount once it has.  (The incremental update visits every
+// triangle a deleted edge closes, with atomics on counts shared by hub edges.)
 constexpr int64_t kRecountShareInv = 4;  // one quarter
 
 kz_status sparse_kernelize_support(kz_graph g, const kz_options &opt, cudaStream_t s) {
@@ -355,19 +305,28 @@ kz_status sparse_kernelize_support(kz_graph g, const kz_options &opt, cudaStream
   const int64_t max_sweeps = opt.max_sweeps > 0 ? opt.max_sweeps : (int64_t)g->n + g->m + 1;
   SupportBufs *b = nullptr;
   KZ_TRY(support_alloc(g, s, b));
-  support_begin_kernel<<<1, 1, 0, s>>>(g->st, max_sweeps, g->n == 0 ? 1 : 0);
-  KZ_CUDA_TRY(cudaGetLastError());
+  KZ_TRY(sparse_begin(g, max_sweeps, s));
   if (g->n == 0) return KZ_OK;
+  // heavy sweeps as plain passes; a remnant that fits bitset rows ends there
+  int64_t live_edges = 0;
+  for (;;) {
+    SparseReport r;
+    KZ_TRY(sparse_one_pass(g, max_sweeps, s, &r));
+    if (!r.cont) return KZ_OK;
+    bool done = false;
+    KZ_TRY(sparse_finish_small(g, max_sweeps, r, s, &done));
+    if (done) return KZ_OK;
+    live_edges = r.live;
+    if ((r.live_before - r.live) * kRecountShareInv <= r.live_before) break;
+  }
   const int grid = 8 * sms_of_device(), threads = 256;
   const int64_t n = g->n, m = g->m;
   const int k = g->k;
-  const int c = g->sp_cur;
-  uint8_t *elive = g->sp_elive[c], *vlive = g->sp_vlive[c];
+  uint8_t *elive = g->sp_elive, *vlive = g->sp_vlive;
   KZ_CUDA_TRY(cudaMemsetAsync(b->dcount, 0, 4, s));
-  // counts of the live graph; the compacted live rows (buffer c ^ 1) serve
-  // the incremental updates until the next recount (dead entries skipped)
-  int64_t live_edges = 0;
-  KZ_TRY(support_recount(g, b, s, &live_edges));
+  // counts of the live graph; the working rows serve the incremental updates
+  // until the next recount (dead entries skipped)
+  KZ_TRY(support_recount(g, b, s));
   for (;;) {
     support_rule_kernel<<<grid, threads, 0, s>>>(g->sp_eu, g->sp_ev, g->sp_col, elive, vlive, m, (int32_t)n, k,
                                                  b->cnt_e, b->cnt_v, b->edirty, b->vdirty, b->edel, b->vdel,
@@ -388,12 +347,12 @@ kz_status sparse_kernelize_support(kz_graph g, const kz_options &opt, cudaStream
     if ((int64_t)deleted * kRecountShareInv > live_edges) {
       support_apply_kernel<<<grid, threads, 0, s>>>(elive, vlive, b->edel, b->vdel, m, (int32_t)n, b->dcount);
       KZ_CUDA_TRY(cudaGetLastError());
-      KZ_TRY(support_recount(g, b, s, &live_edges));
+      live_edges -= (int64_t)deleted;
+      KZ_TRY(support_recount(g, b, s));
       continue;
     }
-    const int nx = c ^ 1;  // the compacted rows of the last recount
-    support_update_kernel<<<grid, threads, 0, s>>>(g->sp_eu, g->sp_ev, g->sp_col, g->sp_row[nx], g->sp_adj[nx],
-                                                   g->sp_eid[nx], elive, b->edel, b->dlist, b->dcount, k, b->cnt_e,
+    support_update_kernel<<<grid, threads, 0, s>>>(g->sp_eu, g->sp_ev, g->sp_col, g->sp_row0, g->sp_len, g->sp_adj,
+                                                   g->sp_eid, elive, b->edel, b->dlist, b->dcount, k, b->cnt_e,
                                                    b->cnt_v, b->edirty, b->vdirty);
     support_apply_kernel<<<grid, threads, 0, s>>>(elive, vlive, b->edel, b->vdel, m, (int32_t)n, b->dcount);
     KZ_CUDA_TRY(cudaGetLastError());
