@@ -261,24 +261,25 @@ __global__ void __launch_bounds__(kThreads, 2) pair_kernel(const __grid_constant
 
 // The lists: one warp per block of v's walks the tiles of lower classes; a
 // lane's entries are its v's neighbours in the tile (vertex i of the tile's
-// block b as 32 b + i), two to a word, padded with kPad to the longest list
-// of the block.  pos[b] is block b's word in a row (rows of `stride` words).
+// block b as 32 b + i), two to a word, padded to the longest list of the block
+// with the index past the tile's rows.  pos[b] is block b's word in a row (rows of `stride` words).
 // FILL = false only adds up the rows the lists take.
 template <bool FILL>
 __global__ void __launch_bounds__(256) lists_kernel(const uint32_t *__restrict__ rows, int64_t stride,
                                                     const int64_t *__restrict__ pos,
                                                     const BlockDesc *__restrict__ blocks,
                                                     const int32_t *__restrict__ boff, int32_t nb, int32_t n_tiles,
-                                                    ListRef *__restrict__ refs, uint32_t *__restrict__ lists,
+                                                    int32_t tile_blocks, ListRef *__restrict__ refs, uint32_t *__restrict__ lists,
                                                     unsigned long long *cursor, unsigned long long *n_tests) {
   const int lane = threadIdx.x & 31;
   const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const uint32_t pad = 32u * (uint32_t)tile_blocks;
   unsigned long long tests = 0;
   for (int64_t job = warp0; job < (int64_t)nb * n_tiles; job += warps) {
     const int tile = (int)(job / nb), y = (int)(job - (int64_t)tile * nb);
     const BlockDesc Y = blocks[y];
-    const int b0 = tile * kTileBlocks, b1 = min(b0 + kTileBlocks, boff[Y.c]);
+    const int b0 = tile * tile_blocks, b1 = min(b0 + tile_blocks, boff[Y.c]);
     const uint32_t *row = rows + (int64_t)(Y.base + min(lane, Y.size - 1)) * stride;
     int deg = 0;
     if (lane < Y.size)
@@ -301,16 +302,238 @@ __global__ void __launch_bounds__(256) lists_kernel(const uint32_t *__restrict__
             e++;
           }
       if (e & 1) {
-        out[(e >> 1) * 32] = held | kPad << 16;
+        out[(e >> 1) * 32] = held | pad << 16;
         e++;
       }
-      for (uint32_t i = e >> 1; i < n2; i++) out[i * 32] = kPad | kPad << 16;
+      for (uint32_t i = e >> 1; i < n2; i++) out[i * 32] = pad | pad << 16;
     }
   }
   if constexpr (FILL) {
     for (int o = 16; o > 0; o >>= 1) tests += __shfl_down_sync(0xffffffffu, tests, o);
     if (lane == 0 && tests) atomicAdd(n_tests, tests);
   }
+}
+
+// ---------------------------------------------------------------------------
+// Passes after the first of a run: every test remembers a witness.
+//
+// hint[class][list row][lane] names, for both entries, the word of the class
+// in which the pair last shared a bit.  A pass looks at that one word of both
+// rows and searches the class only when its bits are gone, so a test costs one
+// random and one conflict-free 4-byte shared load (about 4.5 wavefronts for 32
+// tests) whatever the class length, where pair_kernel reads W words.  Witnesses
+// live as long as a run's lists do: a deleted edge's entry becomes padding, and
+// once three tenths of the listed edges are gone the lists are built anew with
+// every hint at word 0.
+//
+// A job is one class, one tile of u's (all its words of the class staged) and
+// a range of v blocks; a warp holds its block's words transposed, [word][lane].
+// Bound by shared-memory wavefronts (the random word of u above all) and by
+// the 2 bytes of list and 1 of hint a test reads.  Measured at n = 32768,
+// k = 24, p = 0.07: 2.9 ms the first pass with hints, 2.1 ms the fiftieth, where
+// pair_kernel takes 4.6; the pass that finds the hints takes 16 (every test
+// searches), so a run of 52 passes goes from 244 to 144 ms, one of 18 at
+// n = 16384 from 17.2 to 13.8, and runs of 10 gain 3 to 5%.  Runs of two passes,
+// the common kind, keep pair_kernel.  Padding tested as a row of ones instead
+// of masked: 156; list rows of four entries: 155.
+// ---------------------------------------------------------------------------
+
+constexpr int kHintQueue = 12;
+constexpr int kHintAhead = 4;
+constexpr size_t kHintSmem = 225 * 1024;
+constexpr double kHintRebuild = 0.7;  // share of the listed edges still alive below which lists are rebuilt
+
+struct HintArgs {
+  const uint32_t *cm;
+  uint32_t *Edel;
+  const BlockDesc *blocks;
+  const ListRef *refs;
+  uint32_t *lists;
+  uint16_t *hints;          // [class][list row][lane], one byte an entry
+  int64_t hint_rows;        // list rows of a class
+  const int2 *jobs;
+  int32_t n_jobs, span, tile_blocks;
+  int32_t nb, k, ldw, Rp;
+  int64_t cls;
+  unsigned long long *counts;
+  unsigned int *queue;
+};
+
+__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+  return v;
+}
+
+// The queued tests of the warp's lanes, searched over the whole class: a new
+// hint, or a failing edge.
+static __device__ __noinline__ void search_class(const HintArgs &p, const uint32_t *queue, int stride, int cnt,
+                                                 const BlockDesc *tile, uint32_t rows_addr, uint32_t vt_addr, int c,
+                                                 uint32_t first, int v, const BlockDesc Y, unsigned int &fails) {
+  const int lane = threadIdx.x & 31;
+  const int quads = p.Rp >> 2;
+  // every lane walks its own queue, one 16-byte chunk a step, so lanes with
+  // short searches move on to their next test
+  uint32_t e = 0, row = 0;
+  for (int i = -1, q = 0;;) {
+    if (q == 0) {
+      if (++i >= cnt) break;
+      e = queue[i * stride];
+      row = rows_addr + (e & 0xffffu) * (uint32_t)p.Rp * 4u;
+    }
+    const uint4 a = lds128(row + 16 * q);
+    const uint32_t vw = vt_addr + 512 * q;
+    const uint32_t m0 = a.x & lds32(vw), m1 = a.y & lds32(vw + 128), m2 = a.z & lds32(vw + 256),
+                   m3 = a.w & lds32(vw + 384);
+    const bool hit = (m0 | m1 | m2 | m3) != 0u;
+    if (!hit && ++q < quads) continue;
+    const uint32_t idx = e & 0xffffu, place = e >> 16;
+    const int64_t slot = (((int64_t)first + (place >> 1)) * 32 + lane) * 2 + (place & 1);
+    if (hit) {
+      reinterpret_cast<uint8_t *>(p.hints + c * p.hint_rows * 32)[slot] = (uint8_t)(4 * q + (m0 ? 0 : m1 ? 1 : m2 ? 2 : 3));
+    } else {
+      // (other classes' CTAs may read the entry meanwhile: the edge fails either way)
+      reinterpret_cast<uint16_t *>(p.lists)[slot] = (uint16_t)(32 * p.tile_blocks);
+      const BlockDesc B = tile[idx >> 5];
+      const int u = B.base + (int)(idx & 31);
+      const uint32_t bu = 1u << (idx & 31);
+      const uint32_t old = atomicOr(&p.Edel[(int64_t)v * p.ldw + B.r * p.k + B.c], bu);
+      atomicOr(&p.Edel[(int64_t)u * p.ldw + Y.r * p.k + Y.c], 1u << lane);
+      fails += (old & bu) ? 0u : 1u;
+    }
+    q = 0;
+  }
+  __syncwarp();
+}
+
+template <int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, 1) hint_kernel(const __grid_constant__ HintArgs p) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ BlockDesc s_tile[kTileBlocks];
+  __shared__ unsigned int s_job, s_next;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int Rp = p.Rp, quads = Rp >> 2, tile_rows = 32 * p.tile_blocks;
+  uint32_t *rows = reinterpret_cast<uint32_t *>(smem);
+  uint32_t *vt = rows + (size_t)tile_rows * Rp + (size_t)warp * Rp * 32 + lane;
+  uint32_t *queue = rows + (size_t)tile_rows * Rp + (size_t)WARPS * Rp * 32 + t;
+  const uint32_t rows_addr = smem_addr(rows), vt_addr = smem_addr(vt);
+  const uint32_t row_bytes = (uint32_t)Rp * 4u, last_row = (uint32_t)tile_rows - 1u;
+  unsigned int fails = 0;
+  for (;;) {
+    __syncthreads();  // the previous job's rows are no longer read
+    if (t == 0) {
+      s_job = atomicAdd(p.queue, 1u);
+      s_next = 0;
+    }
+    __syncthreads();
+    const unsigned int j = s_job;
+    if (j >= (unsigned int)p.n_jobs * (unsigned int)p.k) break;
+    const int2 job = p.jobs[j % (unsigned int)p.n_jobs];
+    const int c = (int)(j / (unsigned int)p.n_jobs);
+    if (t < p.tile_blocks) {
+      BlockDesc b = {0, 0, 0, 0};
+      if (job.x * p.tile_blocks + t < p.nb) b = p.blocks[job.x * p.tile_blocks + t];
+      s_tile[t] = b;
+    }
+    __syncthreads();
+    const uint32_t *cmc = p.cm + c * p.cls;
+    for (int i = t; i < tile_rows * quads; i += 32 * WARPS) {
+      const int row = i / quads, q = i - row * quads;
+      const BlockDesc B = s_tile[row >> 5];
+      if ((row & 31) >= B.size) continue;
+      uint32_t *dst = rows + (size_t)row * Rp + 4 * q;
+      if (B.c == c)  // not a class the pair needs: v itself has u in it
+        *reinterpret_cast<uint4 *>(dst) = make_uint4(~0u, ~0u, ~0u, ~0u);
+      else
+        cp_async16(dst, cmc + (int64_t)(B.base + (row & 31)) * Rp + 4 * q);
+    }
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
+    const int y_end = min(job.y + p.span, p.nb);
+    auto take = [&]() { return job.y + (int)__shfl_sync(0xffffffffu, lane == 0 ? atomicAdd(&s_next, 1u) : 0u, 0); };
+    int yb = take();
+    ListRef ref = {0, 0};
+    BlockDesc Y = {0, 0, 0, 0};
+    if (yb < y_end) {
+      ref = p.refs[(int64_t)job.x * p.nb + yb];
+      Y = p.blocks[yb];
+    }
+    while (yb < y_end) {
+      const uint32_t first = ref.first;
+      const int n2 = Y.c == c ? 0 : (int)ref.rows;
+      const BlockDesc Yc = Y;
+      // the next block's list and place are on their way meanwhile
+      yb = take();
+      if (yb < y_end) {
+        ref = p.refs[(int64_t)job.x * p.nb + yb];
+        Y = p.blocks[yb];
+      }
+      if (n2 == 0) continue;
+      const uint32_t *lp = p.lists + (int64_t)first * 32 + lane;
+      const uint16_t *hp = p.hints + (c * p.hint_rows + (int64_t)first) * 32 + lane;
+      const uint32_t pads = (uint32_t)tile_rows * 0x10001u;
+      // list rows and hints kHintAhead steps (of two rows) ahead
+      uint32_t le[kHintAhead][2], lh[kHintAhead][2];
+#pragma unroll
+      for (int d = 0; d < kHintAhead; d++)
+#pragma unroll
+        for (int r = 0; r < 2; r++) {
+          const int i = 2 * d + r;
+          le[d][r] = i < n2 ? lp[i * 32] : pads;
+          lh[d][r] = i < n2 ? hp[i * 32] : 0u;
+        }
+      const int v = Yc.base + min(lane, Yc.size - 1);
+      const uint4 *vrow = reinterpret_cast<const uint4 *>(cmc + (int64_t)v * Rp);
+      __syncwarp();  // the previous block's words are no longer read
+#pragma unroll 4
+      for (int q = 0; q < quads; q++) {
+        const uint4 x = vrow[q];
+        vt[128 * q] = x.x;
+        vt[128 * q + 32] = x.y;
+        vt[128 * q + 64] = x.z;
+        vt[128 * q + 96] = x.w;
+      }
+      __syncwarp();
+      int cnt = 0;
+      for (int i0 = 0; i0 < n2; i0 += 2 * kHintAhead) {
+#pragma unroll
+        for (int d = 0; d < kHintAhead; d++) {
+          const int i = i0 + 2 * d;
+          const uint32_t e[4] = {le[d][0] & 0xffffu, le[d][0] >> 16, le[d][1] & 0xffffu, le[d][1] >> 16};
+          const uint32_t h[4] = {lh[d][0] & 0xffu, lh[d][0] >> 8, lh[d][1] & 0xffu, lh[d][1] >> 8};
+#pragma unroll
+          for (int r = 0; r < 2; r++) {
+            const int in = i + 2 * kHintAhead + r;
+            le[d][r] = in < n2 ? lp[in * 32] : pads;
+            lh[d][r] = in < n2 ? hp[in * 32] : 0u;
+          }
+          bool miss[4];
+          bool any = false;
+#pragma unroll
+          for (int x = 0; x < 4; x++) {
+            const uint32_t wu = lds32(rows_addr + mad(min(e[x], last_row), row_bytes, h[x] * 4u));
+            const uint32_t wv = lds32(vt_addr + h[x] * 128u);
+            miss[x] = (wu & wv) == 0u && e[x] <= last_row;
+            any |= miss[x];
+          }
+          if (__any_sync(0xffffffffu, any)) {
+#pragma unroll
+            for (int x = 0; x < 4; x++)
+              if (miss[x]) queue[cnt++ * (32 * WARPS)] = e[x] | (uint32_t)(2 * i + x) << 16;
+            if (__any_sync(0xffffffffu, cnt > kHintQueue - 4)) {
+              search_class(p, queue, 32 * WARPS, cnt, s_tile, rows_addr, vt_addr, c, first, v, Yc, fails);
+              cnt = 0;
+            }
+          }
+        }
+      }
+      if (__any_sync(0xffffffffu, cnt > 0))
+        search_class(p, queue, 32 * WARPS, cnt, s_tile, rows_addr, vt_addr, c, first, v, Yc, fails);
+    }
+  }
+  fails = __reduce_add_sync(0xffffffffu, fails);
+  if (lane == 0 && fails) atomicAdd(&p.counts[0], (unsigned long long)fails);
 }
 
 // Class-major copy of the current rows and the vertex rule, one CTA per row:
@@ -377,8 +600,9 @@ __global__ void commit_kernel(const uint4 *__restrict__ A, uint4 *__restrict__ A
 }
 
 // Closes the pass; report[0] = 1 when the run goes on, report[1] = live edges
-// left.
-__global__ void finish_kernel(DevState *st, unsigned long long *counts, long long *report) {
+// left.  known: the live edges, where no list was counted (else negative).
+__global__ void finish_kernel(DevState *st, unsigned long long *counts, long long *report, long long known) {
+  if (known >= 0) counts[1] = (unsigned long long)known;
   const int cont = finish_pass(st, counts[2], counts[0], counts[1]);
   report[0] = cont;
   report[1] = (long long)(counts[1] - (cont ? counts[0] : 0ull));
@@ -418,24 +642,46 @@ struct PairBufs {
   long long *report = nullptr;                  // of the last pass
   unsigned int *queue = nullptr;
   double live = 0;                              // live edges, as far as the host knows
+  // passes with hints
+  int32_t hint_tile = 0, hint_tiles = 0, hint_warps = 0, hint_span = 0, n_hint_jobs = 0;
+  std::vector<int2> hint_jobs_host;
+  uint8_t *hint_mem = nullptr;  // of the run in progress; the four below lie in it
+  size_t hint_bytes = 0;
+  int2 *hint_jobs = nullptr;
+  ListRef *hint_refs = nullptr;
+  uint32_t *hint_lists = nullptr;
+  uint16_t *hints = nullptr;
+  int64_t hint_rows = 0;
+  bool hint_off = false;   // not for this run
+  double hint_listed = 0;  // live edges when the lists in use were built (0: none)
 };
+
+// Jobs (tile, first block of v's) of `span` blocks of v's each: a tile's words
+// are staged once per job and class group, so long jobs stage less, but there
+// should be about `want` jobs times classes, and a block for every warp.
+static void plan_jobs(kz_graph g, int tile_blocks, int warps, int want, int32_t *span,
+                      std::vector<int2> &jobs) {
+  const int nb = (int)g->blocks.size(), tiles = (nb + tile_blocks - 1) / tile_blocks;
+  std::vector<int> begin((size_t)tiles, 0);
+  int64_t pairs = 0;
+  for (int t = 0; t < tiles; t++) {
+    int y = 0;
+    while (y < nb && g->boff[g->blocks[y].c] <= t * tile_blocks) y++;
+    begin[t] = y;
+    pairs += nb - y;
+  }
+  *span = (int)std::max<int64_t>(warps, std::min<int64_t>(8 * warps, pairs * g->k / want));
+  jobs.clear();
+  for (int t = 0; t < tiles; t++)
+    for (int y = begin[t]; y < nb; y += *span) jobs.push_back(make_int2(t, y));
+}
 
 static kz_status pairs_prepare(kz_graph g, PairBufs &b, cudaStream_t s) {
   const int nb = (int)g->blocks.size(), sms = sms_p();
   b.Rp = (g->R + 3) / 4 * 4;
   b.n_tiles = (nb + kTileBlocks - 1) / kTileBlocks;
-  // blocks of v's per job: a tile's rows are staged once per job and class
-  // group, so long jobs stage less; enough jobs for every CTA slot four times
-  int64_t pairs = 0;
-  for (int t = 0; t < b.n_tiles; t++)
-    for (int y = 0; y < nb; y++) pairs += g->boff[g->blocks[y].c] > t * kTileBlocks;
-  b.span = (int)std::max<int64_t>(kWarps, std::min<int64_t>(8 * kWarps, pairs * g->k / 4 / (8 * sms)));
   std::vector<int2> jobs;
-  for (int t = 0; t < b.n_tiles; t++) {
-    int y = 0;
-    while (y < nb && g->boff[g->blocks[y].c] <= t * kTileBlocks) y++;
-    for (; y < nb; y += b.span) jobs.push_back(make_int2(t, y));
-  }
+  plan_jobs(g, kTileBlocks, kWarps, 32 * sms, &b.span, jobs);  // a class group is four classes or more
   b.n_jobs = (int32_t)jobs.size();
   std::vector<int32_t> block_of((size_t)std::max(g->n, 1));
   std::vector<int64_t> pos((size_t)2 * std::max(nb, 1));
@@ -471,7 +717,7 @@ static kz_status pairs_prepare(kz_graph g, PairBufs &b, cudaStream_t s) {
   unsigned long long list_rows = 0;
   if (nb > 0) {
     lists_kernel<false><<<16 * sms, 256, 0, s>>>(g->A0, g->ldw, b.pos + nb, g->d_blocks, g->d_boff, nb, b.n_tiles,
-                                                 nullptr, nullptr, b.counts + 3, nullptr);
+                                                 kTileBlocks, nullptr, nullptr, b.counts + 3, nullptr);
     KZ_CUDA_TRY(cudaGetLastError());
   }
   KZ_CUDA_TRY(cudaMemcpyAsync(&list_rows, b.counts + 3, 8, cudaMemcpyDeviceToHost, s));
@@ -513,9 +759,67 @@ static kz_status pairs_buffers(kz_graph g, cudaStream_t s) {
   return KZ_OK;
 }
 
+// The hint pass's tile, lists and hints, for the rest of a run: they are given
+// back when it ends.  A graph whose classes are too short to gain, too long for
+// a byte, or whose hints do not fit stays with pair_kernel (hint_off).
+constexpr int kHintMinWords = 12, kHintMaxWords = 255;
+constexpr size_t kHintBudgetBytes = size_t(8) << 30;
+
+static kz_status hint_buffers(kz_graph g, PairBufs &b, cudaStream_t s) {
+  if (b.hint_mem || b.hint_off) return KZ_OK;
+  b.hint_off = true;
+  if (g->R < kHintMinWords || b.Rp > kHintMaxWords) return KZ_OK;
+  const int nb = (int)g->blocks.size(), sms = sms_p();
+  b.hint_warps = b.Rp <= 48 ? 16 : 8;
+  const size_t fixed = (size_t)b.hint_warps * (b.Rp * 128 + kHintQueue * 128);
+  if (fixed + (size_t)b.Rp * 128 > kHintSmem) return KZ_OK;
+  b.hint_tile = (int)std::min<size_t>(kTileBlocks, (kHintSmem - fixed) / ((size_t)b.Rp * 128));
+  if (b.hint_tile < 4) return KZ_OK;  // lists of a few entries
+  b.hint_tiles = (nb + b.hint_tile - 1) / b.hint_tile;
+  if (b.hint_jobs_host.empty()) plan_jobs(g, b.hint_tile, b.hint_warps, 8 * sms, &b.hint_span, b.hint_jobs_host);
+  b.n_hint_jobs = (int32_t)b.hint_jobs_host.size();
+  if (b.n_hint_jobs == 0) return KZ_OK;
+  // the lists of this state: a later one of the run, with fewer edges, takes no
+  // more rows
+  unsigned long long rows = 0;
+  KZ_CUDA_TRY(cudaMemsetAsync(b.counts + 3, 0, 8, s));
+  lists_kernel<false><<<16 * sms, 256, 0, s>>>(b.cm, b.Rp, b.pos, g->d_blocks, g->d_boff, nb, b.hint_tiles,
+                                               b.hint_tile, nullptr, nullptr, b.counts + 3, nullptr);
+  KZ_CUDA_TRY(cudaGetLastError());
+  KZ_CUDA_TRY(cudaMemcpyAsync(&rows, b.counts + 3, 8, cudaMemcpyDeviceToHost, s));
+  KZ_CUDA_TRY(cudaStreamSynchronize(s));
+  const auto part = [](size_t bytes) { return (bytes + 255) & ~(size_t)255; };
+  const size_t jobs = part(sizeof(int2) * b.n_hint_jobs), refs = part(sizeof(ListRef) * b.hint_tiles * nb);
+  const size_t lists = part((size_t)rows * 128), hints = part((size_t)rows * 64 * g->k);
+  if (rows == 0 || rows > UINT32_MAX || lists + hints > kHintBudgetBytes) return KZ_OK;
+  b.hint_bytes = jobs + refs + lists + hints;
+  b.hint_mem = static_cast<uint8_t *>(dev_alloc(b.hint_bytes, s));
+  if (!b.hint_mem) return KZ_OK;  // the passes stay with pair_kernel
+  b.hint_jobs = reinterpret_cast<int2 *>(b.hint_mem);
+  b.hint_refs = reinterpret_cast<ListRef *>(b.hint_mem + jobs);
+  b.hint_lists = reinterpret_cast<uint32_t *>(b.hint_mem + jobs + refs);
+  b.hints = reinterpret_cast<uint16_t *>(b.hint_mem + jobs + refs + lists);
+  b.hint_rows = (int64_t)rows;
+  KZ_CUDA_TRY(cudaMemcpyAsync(b.hint_jobs, b.hint_jobs_host.data(), sizeof(int2) * b.n_hint_jobs,
+                              cudaMemcpyHostToDevice, s));
+  for (int w : {8, 16})
+    KZ_CUDA_TRY(cudaFuncSetAttribute(w == 8 ? (const void *)hint_kernel<8> : (const void *)hint_kernel<16>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHintSmem));
+  b.hint_off = false;
+  return KZ_OK;
+}
+
+static void hint_release(PairBufs &b, cudaStream_t s) {
+  if (b.hint_mem) dev_free(b.hint_mem, b.hint_bytes, s);
+  b.hint_mem = nullptr;
+  b.hint_off = false;
+  b.hint_listed = 0;
+}
+
 // One pass from row buffer `cur` into the other; *cont = 1 when it deleted
-// something and the run goes on.
-static kz_status pairs_pass(kz_graph g, int cur, cudaStream_t s, int *cont) {
+// something and the run goes on.  hints: a later pass of a run, whose tests
+// keep their witnesses.
+static kz_status pairs_pass(kz_graph g, int cur, bool hints, cudaStream_t s, int *cont) {
   PairBufs &b = *static_cast<PairBufs *>(g->pairs_bufs);
   const int sms = sms_p(), nb = (int)g->blocks.size();
   const double density = g->m > 0 ? g->density * b.live / (double)g->m : 0.0;
@@ -543,9 +847,48 @@ static kz_status pairs_pass(kz_graph g, int cur, cudaStream_t s, int *cont) {
   rows_kernel<<<std::min(g->n, 16 * sms), kRowThreads, srow, s>>>(
       g->A[cur], b.cm, g->V[cur], g->V[cur ^ 1], g->d_blocks, b.block_of, g->n, g->k, g->R, g->ldw, b.Rp, g->k,
       g->v_sweep, g->st, b.counts, b.queue, b.counts + 3);
-  if (b.n_jobs > 0) {
-    lists_kernel<true><<<16 * sms, 256, 0, s>>>(b.cm, b.Rp, b.pos, g->d_blocks, g->d_boff, nb, b.n_tiles, b.refs,
-                                                b.lists, b.counts + 3, b.counts + 1);
+  bool hinted = hints && b.n_jobs > 0;
+  if (hinted) {
+    KZ_TRY(hint_buffers(g, b, s));
+    hinted = !b.hint_off;
+  }
+  long long known = -1;
+  if (hinted) {
+    if (b.hint_listed > 0 && b.live >= kHintRebuild * b.hint_listed) {
+      known = (long long)b.live;
+    } else {
+      KZ_CUDA_TRY(cudaMemsetAsync(b.counts + 3, 0, 8, s));
+      lists_kernel<true><<<16 * sms, 256, 0, s>>>(b.cm, b.Rp, b.pos, g->d_blocks, g->d_boff, nb, b.hint_tiles,
+                                                  b.hint_tile, b.hint_refs, b.hint_lists, b.counts + 3, b.counts + 1);
+      KZ_CUDA_TRY(cudaMemsetAsync(b.hints, 0, (size_t)b.hint_rows * 64 * g->k, s));
+      b.hint_listed = b.live;
+    }
+    HintArgs h;
+    h.cm = b.cm;
+    h.Edel = b.Edel;
+    h.blocks = g->d_blocks;
+    h.refs = b.hint_refs;
+    h.lists = b.hint_lists;
+    h.hints = b.hints;
+    h.hint_rows = b.hint_rows;
+    h.jobs = b.hint_jobs;
+    h.n_jobs = b.n_hint_jobs;
+    h.span = b.hint_span;
+    h.tile_blocks = b.hint_tile;
+    h.nb = nb;
+    h.k = g->k;
+    h.ldw = g->ldw;
+    h.Rp = b.Rp;
+    h.cls = a.cls;
+    h.counts = b.counts;
+    h.queue = b.queue;
+    const size_t smem = (size_t)b.hint_tile * b.Rp * 128 + (size_t)b.hint_warps * (b.Rp * 128 + kHintQueue * 128);
+    const int grid = (int)std::min<int64_t>((int64_t)b.n_hint_jobs * g->k, sms);
+    if (b.hint_warps == 16) hint_kernel<16><<<grid, 512, smem, s>>>(h);
+    else hint_kernel<8><<<grid, 256, smem, s>>>(h);
+  } else if (b.n_jobs > 0) {
+    lists_kernel<true><<<16 * sms, 256, 0, s>>>(b.cm, b.Rp, b.pos, g->d_blocks, g->d_boff, nb, b.n_tiles,
+                                                kTileBlocks, b.refs, b.lists, b.counts + 3, b.counts + 1);
     const int64_t work = (int64_t)a.n_jobs * a.n_groups;
     pair_fn(W)<<<(int)std::min<int64_t>(work, 2 * sms), kThreads, kSmemBytes, s>>>(a);
   }
@@ -553,7 +896,7 @@ static kz_status pairs_pass(kz_graph g, int cur, cudaStream_t s, int *cont) {
   commit_kernel<<<(int)std::min<int64_t>((quads + 255) / 256, 16 * sms), 256, 0, s>>>(
       reinterpret_cast<const uint4 *>(g->A[cur]), reinterpret_cast<uint4 *>(g->A[cur ^ 1]),
       reinterpret_cast<uint4 *>(b.Edel), quads);
-  finish_kernel<<<1, 1, 0, s>>>(g->st, b.counts, b.report);
+  finish_kernel<<<1, 1, 0, s>>>(g->st, b.counts, b.report, known);
   KZ_CUDA_TRY(cudaGetLastError());
   long long report[2] = {0, 0};
   KZ_CUDA_TRY(cudaMemcpyAsync(report, b.report, sizeof(report), cudaMemcpyDeviceToHost, s));
@@ -577,7 +920,7 @@ kz_status pairs_one_pass(kz_graph g, cudaStream_t s, int *cont) {
   KZ_TRY(pairs_buffers(g, s));
   int cur = 0;
   KZ_TRY(current_buffer(g, s, &cur));
-  return pairs_pass(g, cur, s, cont);
+  return pairs_pass(g, cur, false, s, cont);
 }
 
 kz_status pairs_kernelize(kz_graph g, const kz_options &opt, cudaStream_t s) {
@@ -585,11 +928,16 @@ kz_status pairs_kernelize(kz_graph g, const kz_options &opt, cudaStream_t s) {
   KZ_TRY(pairs_buffers(g, s));
   KZ_TRY(bitset_begin_run(g, max_sweeps, s));
   if (g->n == 0) return KZ_OK;
-  static_cast<PairBufs *>(g->pairs_bufs)->live = (double)g->m;  // the state may have been reset
+  PairBufs &b = *static_cast<PairBufs *>(g->pairs_bufs);
+  b.live = (double)g->m;  // the state may have been reset
   int cur = 0;
   KZ_TRY(current_buffer(g, s, &cur));
-  for (int cont = 1; cont; cur ^= 1) KZ_TRY(pairs_pass(g, cur, s, &cont));
-  return KZ_OK;
+  // a run that reaches a third pass is a cascade of many, as a rule
+  int pass = 0;
+  kz_status rc = KZ_OK;
+  for (int cont = 1; cont && rc == KZ_OK; cur ^= 1) rc = pairs_pass(g, cur, pass++ >= 2, s, &cont);
+  hint_release(b, s);
+  return rc;
 }
 
 void pairs_release(kz_graph g) {

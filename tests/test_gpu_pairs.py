@@ -32,6 +32,30 @@ def test_pairs_match_the_bitset_sweep(n, k, p):
     _same(a, gpu_run(g, dense=True, path="bitset"))
 
 
+# long cascades, whose passes from the third on keep witnesses: classes of 14 to
+# 55 words (both block widths), lists rebuilt as edges go, twice on one handle,
+# and a run cut off among those passes and continued
+@pytest.mark.parametrize("n,k,p", [(5200, 12, 0.11), (7001, 11, 0.09), (6200, 4, 0.038), (7000, 4, 0.036),
+                                   (9300, 6, 0.055)])
+def test_long_cascades_match_the_bitset_sweep(n, k, p):
+    g = synth.kpartite(n, k, p, 9400 + n, planted=True)
+    want = gpu_run(g, dense=True, path="bitset")
+    assert want["stats"]["sweeps"] >= 6
+    with kz.KernelGraph.from_synth(g, dense=True) as kg:
+        for _ in range(2):
+            kg.reset().kernelize()
+            alive, edges, st = kg.fetch()
+            assert st["path"] == 4 and np.array_equal(alive, want["alive"]) and np.array_equal(edges, want["edges"])
+            for f in ("sweeps", "passes", "edge_tests", "n_live", "m_live"):
+                assert st[f] == want["stats"][f], f
+        kg.reset().kernelize(max_sweeps=4)
+        assert kg.stats(allow=(kz.KZ_ERR_LIMIT,))["sweeps"] == 4
+        kg.kernelize()
+        alive, edges, _ = kg.fetch()
+        assert np.array_equal(alive, want["alive"]) and np.array_equal(edges, want["edges"])
+    _same(gpu_run(g, dense=True), want)
+
+
 @pytest.mark.parametrize("n,k,p", [(3080, 9, 0.09), (3300, 13, 0.11)])
 def test_pairs_match_the_oracle(n, k, p):
     g = synth.kpartite(n, k, p, 9200 + n, planted=True)
