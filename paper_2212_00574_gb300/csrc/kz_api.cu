@@ -10,6 +10,7 @@
 #include <mutex>
 #include <new>
 #include <numeric>
+#include <thread>
 #include <vector>
 
 #include "kz_internal.cuh"
@@ -122,15 +123,45 @@ kz_status check_colours(int32_t n, int32_t k, const int32_t *colour) {
   return KZ_OK;
 }
 
-kz_status check_edges(int32_t n, const int32_t *colour, int64_t m, const int32_t *edges) {
-  if (m < 0) return KZ_ERR_ARG;
-  if (m > 0 && !edges) return KZ_ERR_ARG;
-  for (int64_t e = 0; e < m; e++) {
+// The verdict on the first wrong edge of [begin, end).
+kz_status first_wrong(int32_t n, const int32_t *colour, const int32_t *edges, int64_t begin, int64_t end) {
+  for (int64_t e = begin; e < end; e++) {
     const int32_t u = edges[2 * e], v = edges[2 * e + 1];
     if (u < 0 || u >= n || v < 0 || v >= n) return KZ_ERR_VERTEX_RANGE;
     if (u == v) return KZ_ERR_SELF_LOOP;
     if (colour[u] == colour[v]) return KZ_ERR_ILLEGAL_COLOURING;
   }
+  return KZ_OK;
+}
+
+// A long list is checked by several threads, each a run of it: the first run
+// with a wrong edge decides.  An edge takes 1.05 ns (6.2 ms of a load with 5.9
+// million, where the device's share is 1.2); eight threads take 0.9 ms, sixteen
+// would 0.64, and a loop without branches takes 1.7 ns an edge.  A thread
+// starts in 20 us, a tenth of what its run of kCheckShare edges takes.
+constexpr int64_t kCheckShare = int64_t(1) << 18;
+constexpr int kCheckThreads = 8;
+
+kz_status check_edges(int32_t n, const int32_t *colour, int64_t m, const int32_t *edges) {
+  if (m < 0) return KZ_ERR_ARG;
+  if (m > 0 && !edges) return KZ_ERR_ARG;
+  const int64_t cores = std::max<int64_t>(std::thread::hardware_concurrency(), 1);
+  const int runs = (int)std::max<int64_t>(1, std::min<int64_t>({m / kCheckShare, cores, kCheckThreads}));
+  kz_status verdict[kCheckThreads];
+  std::thread helper[kCheckThreads];
+  const auto check = [&](int i) { verdict[i] = first_wrong(n, colour, edges, m * i / runs, m * (i + 1) / runs); };
+  for (int i = 1; i < runs; i++) {
+    try {
+      helper[i] = std::thread(check, i);
+    } catch (...) {
+      check(i);  // no thread to be had
+    }
+  }
+  check(0);
+  for (int i = 1; i < runs; i++)
+    if (helper[i].joinable()) helper[i].join();
+  for (int i = 0; i < runs; i++)
+    if (verdict[i] != KZ_OK) return verdict[i];
   return KZ_OK;
 }
 
