@@ -269,6 +269,7 @@ __global__ void rank_kernel(const uint64_t *__restrict__ keys, int32_t n, int32_
 struct Scratch {
   cudaStream_t s;
   std::vector<std::pair<void *, size_t>> held;
+  bool refused = false;
   explicit Scratch(cudaStream_t st) : s(st) {}
   ~Scratch() {
     for (auto &h : held) dev_free(h.first, h.second, s);
@@ -276,8 +277,9 @@ struct Scratch {
   template <class T>
   T *get(size_t count) {
     const size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
-    void *p = dev_alloc(bytes, s);
+    void *p = refused ? nullptr : dev_alloc(bytes, s);
     if (p) held.emplace_back(p, bytes);
+    refused = !p;  // nothing more is asked for then
     return static_cast<T *>(p);
   }
 };
