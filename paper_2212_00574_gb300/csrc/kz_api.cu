@@ -714,45 +714,29 @@ kz_status kz_fetch_kernel_dense(kz_graph g, uint8_t *vertex_alive, uint64_t *adj
     if (stats) *stats = tmp;
     return dev_status;
   }
-  // everything on the stream, one wait at the end: the caller-ordered rows
-  // and vertex flags (gathered on the device), the bit count, the run record
-  const size_t aux = 16 + (size_t)g->n;
-  uint8_t *d_aux = (uint8_t *)dev_alloc(aux, g->stream);
-  kz_status st = d_aux ? KZ_OK : KZ_ERR_OOM;
-  unsigned long long cnt = 0;
-  std::vector<uint8_t> alive((size_t)std::max(g->n, 1));
-  DevState hs;
-  unsigned long long *d_cnt = reinterpret_cast<unsigned long long *>(d_aux);
-  if (st == KZ_OK) st = bitset_fetch_dense(g, adj_bits, row_words, d_aux + 16, d_cnt, g->stream);
-  if (st == KZ_OK && g->n)
-    st = cuda_status(cudaMemcpyAsync(alive.data(), d_aux + 16, (size_t)g->n, cudaMemcpyDeviceToHost, g->stream));
-  if (st == KZ_OK)
-    st = cuda_status(cudaMemcpyAsync(&cnt, d_cnt, 8, cudaMemcpyDeviceToHost, g->stream));
-  if (st == KZ_OK)
-    st = cuda_status(cudaMemcpyAsync(&hs, g->st, offsetof(DevState, trace_dv), cudaMemcpyDeviceToHost, g->stream));
-  if (st == KZ_OK) st = cuda_status(cudaStreamSynchronize(g->stream));
-  if (d_aux) dev_free(d_aux, aux, g->stream);
-  if (st != KZ_OK) return st;
+  std::vector<uint8_t> host;
+  DenseFetch got;
+  KZ_TRY(bitset_fetch_dense(g, adj_bits, row_words, host, &got, g->stream));
   int64_t n_live = 0;
-  for (int32_t v = 0; v < g->n; v++) n_live += alive[v];
-  if (vertex_alive && g->n) memcpy(vertex_alive, alive.data(), (size_t)g->n);
+  for (int32_t v = 0; v < g->n; v++) n_live += got.alive[v];
+  if (vertex_alive && g->n) memcpy(vertex_alive, got.alive, (size_t)g->n);
   if (stats) {
     memset(stats, 0, sizeof(*stats));
     stats->n = g->n;
     stats->m = g->m;
-    stats->sweeps = hs.sweeps;
-    stats->passes = hs.passes;
-    stats->edge_tests = hs.tests;
+    stats->sweeps = got.sweeps;
+    stats->passes = got.passes;
+    stats->edge_tests = got.tests;
     stats->path = g->path_ran;
-    stats->status = hs.status;
+    stats->status = got.status;
     stats->k = g->k;
     stats->clique_k = g->k - g->slack;
     stats->dominance_rounds = g->dom_rounds;
     stats->dominated = (int32_t)g->dom_removed;
     stats->n_live = n_live;
-    stats->m_live = (int64_t)(cnt / 2);
+    stats->m_live = (int64_t)(got.set_bits / 2);
   }
-  return (kz_status)hs.status;
+  return (kz_status)got.status;
 }
 
 kz_status kz_fetch_kernel(kz_graph g, uint8_t *vertex_alive, int32_t *edges_out, int64_t cap,

@@ -192,11 +192,16 @@ kz_status bitset_finish_load(kz_graph g, cudaStream_t s);
 kz_status bitset_reset(kz_graph g, cudaStream_t s);
 kz_status bitset_kernelize(kz_graph g, const kz_options &opt, cudaStream_t s);
 // Caller-ordered dense rows of the current state into host memory (row
-// chunks, each copied while the next is unpacked), vertex flags (bytes, on
-// the device) and the count of set bits (twice the edges, on the device).
-// Asynchronous on s: the caller's wait on s covers every copy.
-kz_status bitset_fetch_dense(kz_graph g, uint64_t *h_out, int64_t row_words, uint8_t *d_alive,
-                             unsigned long long *d_edge_count, cudaStream_t s);
+// chunks, each copied while the next is unpacked), and what DenseFetch names;
+// `host` holds the vertex flags it points to.  Synchronous.
+struct DenseFetch {
+  int64_t sweeps, passes, tests;  // of the last run
+  int32_t status;
+  unsigned long long set_bits;    // in the rows: twice the edges
+  const uint8_t *alive;           // a byte a vertex
+};
+kz_status bitset_fetch_dense(kz_graph g, uint64_t *h_out, int64_t row_words, std::vector<uint8_t> &host,
+                             DenseFetch *got, cudaStream_t s);
 kz_status bitset_vertex_alive(kz_graph g, uint8_t *host_alive, int64_t *n_live);
 
 // One plain multi-CTA sweep pass (no loop graph); *cont = 1 when it deleted
