@@ -856,9 +856,11 @@ __global__ void test_edges_kernel(RowView r, const int2 *__restrict__ work, cons
 
 // Removes the failing edges and the failing vertices (with all their edges)
 // in place, recording each failing vertex's sweep.
+// cm: a class-major copy of the rows to be kept up to date (or null); the list
+// then holds every edge of a failing vertex.
 __global__ void apply_kernel(RowView r, const uint8_t *__restrict__ vfail, const int2 *__restrict__ dead,
                              const unsigned long long *__restrict__ n_dead, int32_t *__restrict__ v_sweep,
-                             const DevState *st) {
+                             const DevState *st, uint32_t *__restrict__ cm, int32_t Rp) {
   const int lane = threadIdx.x & 31;
   const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -868,6 +870,10 @@ __global__ void apply_kernel(RowView r, const uint8_t *__restrict__ vfail, const
     const int cx = r.col[x], cy = r.col[y], ix = x - r.coff[cx], iy = y - r.coff[cy];
     atomicAnd(&r.A[(int64_t)x * r.ldw + (iy >> 5) * r.k + cy], ~(1u << (iy & 31)));
     atomicAnd(&r.A[(int64_t)y * r.ldw + (ix >> 5) * r.k + cx], ~(1u << (ix & 31)));
+    if (cm) {
+      atomicAnd(&cm[((int64_t)x * r.k + cy) * Rp + (iy >> 5)], ~(1u << (iy & 31)));
+      atomicAnd(&cm[((int64_t)y * r.k + cx) * Rp + (ix >> 5)], ~(1u << (ix & 31)));
+    }
   }
   const int64_t warp0 = tid >> 5, warps = stride >> 5;
   const int rk = r.R * r.k;
@@ -964,20 +970,39 @@ constexpr int kRecheckCtasPerSm = 6;
 // passed before the previous sweep.  A failing vertex's edges all fail the
 // edge rule too (no common neighbour can have the colour it lost), so the
 // listed edges are the sweep's whole edge deletion.
+//
+// The vertex rule goes along: a live vertex passed it before the previous
+// sweep, so it fails now only if one of its deleted edges was the last into a
+// class, whose words in cm are then all zero (vfail, n_vfail).  Evaluating the
+// rule of every vertex took 25 us a sweep at n = 16384, k = 24.
 __global__ void __launch_bounds__(256, kRecheckCtasPerSm) recheck_kernel(RowView rold, RowView rnew, const uint32_t *__restrict__ cm, int32_t Rp,
-                               const int2 *__restrict__ dead,
-                               const unsigned long long *__restrict__ n_dead, int64_t q0, int64_t q1, int64_t cap,
+                               const int2 *__restrict__ dead, int64_t q0, int64_t q1, int64_t cap,
                                uint32_t *__restrict__ failed, int2 *__restrict__ out, unsigned long long *n_out,
-                               uint32_t *__restrict__ checked, unsigned long long *n_checked) {
+                               uint32_t *__restrict__ checked, unsigned long long *n_checked,
+                               uint32_t *__restrict__ vfail, unsigned long long *n_vfail) {
   const int lane = threadIdx.x & 31;
   const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = min(min((int64_t)*n_dead, cap), q1);
   const int rk = rold.R * rold.k;
   unsigned int first = 0;
-  for (int64_t q = q0 + warp0; q < total; q += warps) {
+  for (int64_t q = q0 + warp0; q < q1; q += warps) {
     const int2 e = dead[q];
     const int ca = rold.col[e.x], cb = rold.col[e.y];
+    {
+      const uint32_t *wa = cm + ((int64_t)e.x * rnew.k + cb) * Rp, *wb = cm + ((int64_t)e.y * rnew.k + ca) * Rp;
+      uint32_t left_a = 0, left_b = 0;
+      for (int i = lane; i < Rp; i += 32) {
+        left_a |= wa[i];
+        left_b |= wb[i];
+      }
+      left_a = __reduce_or_sync(0xffffffffu, left_a);
+      left_b = __reduce_or_sync(0xffffffffu, left_b);
+      const int x = lane == 0 ? e.x : e.y;
+      if (lane < 2 && (lane == 0 ? left_a : left_b) == 0u && vertex_live(rnew, x)) {
+        const uint32_t byte = 1u << (8 * (x & 3));
+        if (!(atomicOr(&vfail[x >> 2], byte) & byte)) atomicAdd(n_vfail, 1ull);
+      }
+    }
     const uint32_t *ra = rold.A + (int64_t)e.x * rold.ldw, *rb = rold.A + (int64_t)e.y * rold.ldw;
     const uint32_t *na = rnew.A + (int64_t)e.x * rnew.ldw, *nb = rnew.A + (int64_t)e.y * rnew.ldw;
     for (int w = 4 * lane; w < rk; w += 128) {
@@ -1448,7 +1473,7 @@ kz_status learned_kernelize(kz_graph g, const kz_options &opt, int full_path, cu
       KZ_CUDA_TRY(cudaMemsetAsync(b.cnt + 7, 0, sizeof(unsigned long long), s));
       dirty_valid = false;
     }
-    apply_kernel<<<grid, 256, 0, s>>>(r, b.s.vfail, b.dead, b.cnt + 2, g->v_sweep, g->st);
+    apply_kernel<<<grid, 256, 0, s>>>(r, b.s.vfail, b.dead, b.cnt + 2, g->v_sweep, g->st, nullptr, 0);
     learned_finish_kernel<<<1, 1, 0, s>>>(g->st, b.cnt + 3, b.cnt + 2, b.cnt + 1, nullptr);
     KZ_CUDA_TRY(cudaGetLastError());
     round++;
@@ -1495,11 +1520,9 @@ kz_status recheck_kernelize(kz_graph g, const kz_options &opt, int full_path, cu
   const int64_t cap = std::max<int64_t>(g->m, 1);
   const size_t set_bytes = (size_t)g->n * g->ldw * 4;
   const size_t row_bytes = (size_t)g->n * g->ldw * 4, v_bytes = (size_t)g->ldw * 4;
-  unsigned long long h[kCounters];
-  int64_t sweeps = 0;
+  unsigned long long h[4];
   auto read_counts = [&]() -> kz_status {
     KZ_CUDA_TRY(cudaMemcpyAsync(h, b.cnt, sizeof(h), cudaMemcpyDeviceToHost, s));
-    KZ_CUDA_TRY(cudaMemcpyAsync(&sweeps, &g->st->sweeps, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     KZ_CUDA_TRY(cudaStreamSynchronize(s));
     return KZ_OK;
   };
@@ -1511,6 +1534,8 @@ kz_status recheck_kernelize(kz_graph g, const kz_options &opt, int full_path, cu
   double full_ms = -1.0, per_dead_ms = -1.0;
   int cur = 0;
   int2 *dead = b.dead, *fresh = b.work;
+  int64_t n_dead = 0, sweeps = 0;  // of the last sweep; applied so far
+  bool cm_built = false;           // cm holds the rows of buffer cur
   // a full pass, timed; then its deletions listed from the two buffers
   auto full_sweep = [&](int *cont) -> kz_status {
     KZ_CUDA_TRY(cudaEventRecord(ev.a, s));
@@ -1521,46 +1546,53 @@ kz_status recheck_kernelize(kz_graph g, const kz_options &opt, int full_path, cu
     if (ms > 0.0) full_ms = ms;
     if (!*cont) return KZ_OK;
     cur = read_cur(g, s);
+    cm_built = false;
     KZ_CUDA_TRY(cudaMemsetAsync(b.cnt + 2, 0, sizeof(unsigned long long), s));
     diff_dead_kernel<<<grid, 256, 0, s>>>(view_of(g, b, cur ^ 1), g->A[cur & 1], dead, b.cnt + 2, cap);
     KZ_CUDA_TRY(cudaGetLastError());
+    KZ_CUDA_TRY(cudaMemcpyAsync(&sweeps, &g->st->sweeps, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    KZ_TRY(read_counts());
+    n_dead = (int64_t)std::min<unsigned long long>(h[2], (unsigned long long)cap);
     return KZ_OK;
   };
   int cont = 0;
   KZ_TRY(full_sweep(&cont));
   if (!cont) return KZ_OK;  // nothing deleted (or the sweep limit)
   for (;;) {
-    // [0] failures found [1] pairs re-checked [2] deleted by the last sweep [3] failing vertices
-    KZ_TRY(read_counts());
-    const int64_t n_dead = (int64_t)std::min<unsigned long long>(h[2], (unsigned long long)cap);
+    // counters: [0] failures found [1] pairs re-checked [3] failing vertices
     const RowView rnew = view_of(g, b, cur), rold = view_of(g, b, cur ^ 1);
-    bool cm_built = false;
     auto recheck = [&](int64_t q0, int64_t q1) -> kz_status {
       KZ_CUDA_TRY(cudaEventRecord(ev.a, s));
       if (!cm_built) {
         class_major_kernel<<<grid, 256, 0, s>>>(rnew.A, g->n, g->k, g->R, g->ldw, Rp, b.cm);
         cm_built = true;
       }
-      recheck_kernel<<<kRecheckCtasPerSm * sms_now(), 256, 0, s>>>(rold, rnew, b.cm, Rp, dead, b.cnt + 2, q0, q1,
-                                                                    cap, b.pend, fresh, b.cnt + 0, b.dirty,
-                                                                    b.cnt + 1);
+      recheck_kernel<<<kRecheckCtasPerSm * sms_now(), 256, 0, s>>>(rold, rnew, b.cm, Rp, dead, q0, q1, cap, b.pend,
+                                                                    fresh, b.cnt + 0, b.dirty, b.cnt + 1,
+                                                                    reinterpret_cast<uint32_t *>(b.s.vfail),
+                                                                    b.cnt + 3);
       KZ_CUDA_TRY(cudaGetLastError());
       KZ_CUDA_TRY(cudaEventRecord(ev.b, s));
-      KZ_CUDA_TRY(cudaEventSynchronize(ev.b));
-      const double ms = ev.ms();
-      if (ms > 0.0 && q1 - q0 >= 4096) per_dead_ms = ms / (double)(q1 - q0);
       return KZ_OK;
+    };
+    // after a wait for the stream
+    auto time_recheck = [&](int64_t listed) {
+      if (listed < 4096) return;
+      const double ms = ev.ms();
+      if (ms > 0.0) per_dead_ms = ms / (double)listed;
     };
     KZ_CUDA_TRY(cudaMemsetAsync(b.pend, 0, set_bytes, s));
     KZ_CUDA_TRY(cudaMemsetAsync(b.dirty, 0, set_bytes, s));
-    KZ_CUDA_TRY(cudaMemsetAsync(b.cnt, 0, sizeof(unsigned long long) * 2, s));
-    KZ_CUDA_TRY(cudaMemsetAsync(b.cnt + 3, 0, sizeof(unsigned long long), s));
+    KZ_CUDA_TRY(cudaMemsetAsync(b.s.vfail, 0, (size_t)g->n, s));
+    KZ_CUDA_TRY(cudaMemsetAsync(b.cnt, 0, sizeof(unsigned long long) * 4, s));
     bool by_recheck = true;
     int64_t done = 0;
     if (full_ms > 0.0) {
       if (per_dead_ms < 0.0 && n_dead > kRecheckSample) {
         KZ_TRY(recheck(0, kRecheckSample));
         done = kRecheckSample;
+        KZ_CUDA_TRY(cudaEventSynchronize(ev.b));
+        time_recheck(done);
       }
       if (per_dead_ms > 0.0 && (double)(n_dead - done) * per_dead_ms > kRecheckGain * full_ms) by_recheck = false;
     }
@@ -1572,9 +1604,8 @@ kz_status recheck_kernelize(kz_graph g, const kz_options &opt, int full_path, cu
       continue;
     }
     if (done < n_dead) KZ_TRY(recheck(done, n_dead));
-    stats_kernel<<<grid, 256, 0, s>>>(rnew, b.s, 0, b.cnt + 3);
-    KZ_CUDA_TRY(cudaGetLastError());
     KZ_TRY(read_counts());
+    if (done < n_dead) time_recheck(n_dead - done);
     const unsigned long long de = std::min<unsigned long long>(h[0], (unsigned long long)cap), dv = h[3];
     if (de + dv > 0 && sweeps >= max_sweeps) {
       int32_t lim = KZ_ERR_LIMIT;
@@ -1584,18 +1615,21 @@ kz_status recheck_kernelize(kz_graph g, const kz_options &opt, int full_path, cu
     }
     if (de + dv > 0) {
       // the next state in the other buffer: a copy of the current rows with
-      // this sweep's deletions applied
+      // this sweep's deletions applied (to the class-major copy too, which
+      // took 32 us a sweep to build anew at n = 16384, k = 24)
       KZ_CUDA_TRY(cudaMemcpyAsync(g->A[(cur & 1) ^ 1], g->A[cur & 1], row_bytes, cudaMemcpyDeviceToDevice, s));
       KZ_CUDA_TRY(cudaMemcpyAsync(g->V[(cur & 1) ^ 1], g->V[cur & 1], v_bytes, cudaMemcpyDeviceToDevice, s));
-      apply_kernel<<<grid, 256, 0, s>>>(view_of(g, b, cur ^ 1), b.s.vfail, fresh, b.cnt + 0, g->v_sweep, g->st);
+      apply_kernel<<<grid, 256, 0, s>>>(view_of(g, b, cur ^ 1), b.s.vfail, fresh, b.cnt + 0, g->v_sweep, g->st,
+                                        cm_built ? b.cm : nullptr, Rp);
       KZ_CUDA_TRY(cudaGetLastError());
     }
     recheck_finish_kernel<<<1, 1, 0, s>>>(g->st, b.cnt + 3, b.cnt + 0, b.cnt + 1);
     KZ_CUDA_TRY(cudaGetLastError());
     if (de + dv == 0) return KZ_OK;  // the fixpoint: the last sweep broke nothing
     cur ^= 1;
+    sweeps++;
+    n_dead = (int64_t)de;
     std::swap(dead, fresh);
-    KZ_CUDA_TRY(cudaMemcpyAsync(b.cnt + 2, b.cnt + 0, sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
   }
 }
 
