@@ -982,10 +982,14 @@ kz_status bitset_kernelize(kz_graph g, const kz_options &opt, cudaStream_t s) {
   }
   if (g->n > 0 && opt.use_graph == 1) {
     // every pass in one cooperative launch (grid fully resident) after the
-    // run-start kernel.  A graph that fills the GPU launches both as one CUDA
-    // graph (measured 2 us less on C2); a small one launches them directly
-    // (a graph launch was slower there).
-    if (g->plan[form].grid >= sm_count()) {
+    // run-start kernel.  From its second run on, a handle that fills the GPU
+    // launches both as one CUDA graph (measured 2 us less on C2); its first
+    // run, which may be its only one, does not pay for building and releasing
+    // the graph (65 us), and a small graph always launches them directly (a
+    // graph launch was slower there).
+    const bool again = g->ran_before;
+    g->ran_before = true;
+    if (again && g->plan[form].grid >= sm_count()) {
       if (g->run_exec && (g->run_max_sweeps != max_sweeps || g->run_form != form || g->run_slack != g->slack)) {
         cudaGraphExecDestroy(g->run_exec);
         g->run_exec = nullptr;

@@ -162,6 +162,7 @@ struct kz_graph_s {
   // executable CUDA graph of one persistent run: run-start kernel, then the
   // cooperative sweep kernel (built lazily; one launch per kz_kernelize)
   cudaGraphExec_t run_exec = nullptr;
+  bool ran_before = false;  // a persistent run has been launched directly
   int64_t run_max_sweeps = 0;
   int32_t run_form = -1;
   int32_t run_slack = 0;

@@ -617,13 +617,12 @@ static kz_status pack_setup(kz_graph g, cudaStream_t s, PackArgs &a, std::vector
     for (int x = g->coff[c]; x < g->coff[c + 1]; x++) col_new[x] = c;
   // small tables of the packers: carved from the graph's chunks (one
   // allocator call at most), released with the graph
-  int32_t *d_inv = nullptr, *d_col = nullptr, *d_coff = nullptr, *d_err = nullptr;
-  unsigned long long *d_cnt = nullptr;
+  int32_t *d_inv = nullptr, *d_col = nullptr, *d_coff = nullptr;
+  unsigned long long *d_cnt = nullptr;  // edges, error
   const size_t nn = (size_t)std::max(g->n, 1);
   KZ_TRY(graph_alloc(g, &d_inv, nn, s));
   KZ_TRY(graph_alloc(g, &d_col, nn, s));
   KZ_TRY(graph_alloc(g, &d_coff, (size_t)g->k + 1, s));
-  KZ_TRY(graph_alloc(g, &d_err, 4, s));
   KZ_TRY(graph_alloc(g, &d_cnt, 2, s));
   tmp.clear();
   if (g->n) {
@@ -631,7 +630,6 @@ static kz_status pack_setup(kz_graph g, cudaStream_t s, PackArgs &a, std::vector
     KZ_TRY(h2d(d_col, col_new.data(), (size_t)g->n * 4, s));
   }
   KZ_TRY(h2d(d_coff, g->coff.data(), ((size_t)g->k + 1) * 4, s));
-  KZ_CUDA_TRY(cudaMemsetAsync(d_err, 0, 16, s));
   KZ_CUDA_TRY(cudaMemsetAsync(d_cnt, 0, 16, s));
   a.A = g->A0;
   a.ldw = g->ldw;
@@ -640,22 +638,19 @@ static kz_status pack_setup(kz_graph g, cudaStream_t s, PackArgs &a, std::vector
   a.col = d_col;
   a.coff = d_coff;
   a.edge_count = d_cnt;
-  a.error = d_err;
+  a.error = reinterpret_cast<int32_t *>(d_cnt + 1);
   return KZ_OK;
 }
 
 static kz_status pack_finish(kz_graph g, cudaStream_t s, PackArgs &a, std::vector<void *> &tmp) {
-  int32_t err = 0;
-  unsigned long long cnt = 0;
-  cudaError_t e1 = cudaMemcpyAsync(&err, a.error, 4, cudaMemcpyDeviceToHost, s);
-  cudaError_t e2 = cudaMemcpyAsync(&cnt, a.edge_count, 8, cudaMemcpyDeviceToHost, s);
-  cudaError_t e3 = cudaStreamSynchronize(s);
+  unsigned long long h[2] = {0, 0};  // edges, error
+  cudaError_t e1 = cudaMemcpyAsync(h, a.edge_count, sizeof(h), cudaMemcpyDeviceToHost, s);
+  cudaError_t e2 = cudaStreamSynchronize(s);
   tmp.clear();
   if (e1 != cudaSuccess) return cuda_status(e1);
   if (e2 != cudaSuccess) return cuda_status(e2);
-  if (e3 != cudaSuccess) return cuda_status(e3);
-  if (err) return (kz_status)err;
-  g->m = (int64_t)cnt;
+  if (h[1]) return (kz_status)h[1];
+  g->m = (int64_t)h[0];
   return KZ_OK;
 }
 
