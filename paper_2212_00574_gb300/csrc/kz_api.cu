@@ -229,23 +229,7 @@ kz_status load_common(int32_t n, int32_t k, const int32_t *colour, void *stream,
   const size_t bitset_bytes = (size_t)3 * g->n * g->ldw * 4;
   const bool want_bitset = lay == KZ_OK && bitset_bytes <= kBitsetBudgetBytes;
   if (st == KZ_OK && want_bitset) {
-    st = graph_alloc(g, &g->d_perm, (size_t)std::max(n, 1), g->stream);
-    if (st == KZ_OK) st = graph_alloc(g, &g->d_inv, (size_t)std::max(n, 1), g->stream);
-    if (st == KZ_OK) st = graph_alloc(g, &g->d_cpos, (size_t)std::max(n, 1), g->stream);
-    if (st == KZ_OK && n > 0)
-      st = h2d(g->d_perm, g->perm.data(), sizeof(int32_t) * n, g->stream);
-    if (st == KZ_OK && n > 0)
-      st = h2d(g->d_inv, g->inv.data(), sizeof(int32_t) * n, g->stream);
-    if (st == KZ_OK && n > 0) {
-      // position of every caller vertex inside a row of the block-plane layout
-      std::vector<int32_t> cpos((size_t)n);
-      for (int c = 0; c < k; c++)
-        for (int x = g->coff[c]; x < g->coff[c + 1]; x++) {
-          const int ix = x - g->coff[c];
-          cpos[g->perm[x]] = ((((ix >> 5) * k) + c) << 5) | (ix & 31);
-        }
-      st = h2d(g->d_cpos, cpos.data(), sizeof(int32_t) * n, g->stream);
-    }
+    st = bitset_upload_tables(g, g->stream);
     if (st == KZ_OK) st = pack(g);
     if (st == KZ_OK) st = bitset_finish_load(g, g->stream);
     if (st == KZ_OK) g->has_bitset = true;

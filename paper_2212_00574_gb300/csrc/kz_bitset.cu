@@ -161,10 +161,51 @@ __global__ void fill_units_kernel(int2 *__restrict__ units, const int32_t *__res
   }
 }
 
-__global__ void init_vlive_kernel(uint32_t *V, const BlockDesc *blocks, int nb, int k) {
-  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x) {
-    const BlockDesc d = blocks[b];
-    V[d.r * k + d.c] = d.size >= 32 ? 0xffffffffu : ((1u << d.size) - 1u);
+// Everything the layout fixes, from the class and block offsets and the
+// relabelling: per vertex its new id, its class and its position in a row, per
+// block its place, and the live masks of the loaded graph.  Built here, the
+// load copies one table to the device instead of ten and the host fills none of
+// the others: 25 us of a load, kernel and fetch of n = 300 (191 to 167,
+// 271 to 247 at n = 4096), 70 at n = 32768.
+__global__ void __launch_bounds__(256) tables_kernel(const int32_t *__restrict__ perm, const int32_t *__restrict__ coff,
+                                                     const int32_t *__restrict__ boff, int32_t n, int32_t k,
+                                                     int32_t nb, int32_t ldw, int32_t *__restrict__ inv,
+                                                     int32_t *__restrict__ col, int32_t *__restrict__ cpos,
+                                                     BlockDesc *__restrict__ blocks, uint32_t *__restrict__ V0) {
+  __shared__ int32_t sc[65], sb[65];
+  for (int i = threadIdx.x; i <= k; i += blockDim.x) {
+    sc[i] = coff[i];
+    sb[i] = boff[i];
+  }
+  __syncthreads();
+  // the last class that begins at or before i (empty classes begin where the next one does)
+  auto class_of = [k](const int32_t *off, int i) {
+    int lo = 0, hi = k - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (off[mid] <= i) lo = mid;
+      else hi = mid - 1;
+    }
+    return lo;
+  };
+  const int i0 = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+  for (int x = i0; x < n; x += step) {
+    const int c = class_of(sc, x), v = perm[x], ix = x - sc[c];
+    inv[v] = x;
+    col[x] = c;
+    cpos[v] = ((((ix >> 5) * k) + c) << 5) | (ix & 31);
+  }
+  for (int i = i0; i < nb; i += step) {
+    BlockDesc b;
+    b.c = class_of(sb, i);
+    b.r = i - sb[b.c];
+    b.base = sc[b.c] + 32 * b.r;
+    b.size = min(32, sc[b.c + 1] - b.base);
+    blocks[i] = b;
+  }
+  for (int w = i0; w < ldw; w += step) {
+    const int c = w % k, left = sc[c + 1] - sc[c] - 32 * (w / k);
+    V0[w] = left >= 32 ? 0xffffffffu : left > 0 ? (1u << left) - 1u : 0u;
   }
 }
 
@@ -656,23 +697,44 @@ static int sm_count() {
 
 static kz_status ensure_plan(kz_graph g, int form, cudaStream_t s);
 
-kz_status bitset_finish_load(kz_graph g, cudaStream_t s) {
-  const int nb = (int)g->blocks.size();
+kz_status bitset_upload_tables(kz_graph g, cudaStream_t s) {
+  const int n = g->n, k = g->k, nb = (int)g->blocks.size();
+  // the relabelling, the class and block offsets, the classes' rounds, and the
+  // prefix of the block pairs (x, y) with class(x) < class(y)
+  const auto part = [](int64_t count) { return (size_t)((count + 63) & ~int64_t(63)); };
+  const size_t at_coff = part(n), at_boff = at_coff + part(k + 1), at_rounds = at_boff + part(k + 1);
+  const size_t at_poff = at_rounds + part(k), total = at_poff + part(nb + 1);
+  std::vector<int32_t> h(total, 0);
+  std::copy(g->perm.begin(), g->perm.end(), h.begin());
+  std::copy(g->coff.begin(), g->coff.end(), h.begin() + at_coff);
+  std::copy(g->boff.begin(), g->boff.end(), h.begin() + at_boff);
+  std::copy(g->rounds.begin(), g->rounds.end(), h.begin() + at_rounds);
+  int32_t *poff = h.data() + at_poff;
+  for (int x = 0; x < nb; x++) poff[x + 1] = poff[x] + (nb - g->boff[g->blocks[x].c + 1]);
+  g->n_pairs = poff[nb];
+  int32_t *d = nullptr;
+  KZ_TRY(graph_alloc(g, &d, total, s));
+  KZ_TRY(graph_alloc(g, &g->d_inv, (size_t)std::max(n, 1), s));
+  KZ_TRY(graph_alloc(g, &g->d_cpos, (size_t)std::max(n, 1), s));
+  KZ_TRY(graph_alloc(g, &g->d_col, (size_t)std::max(n, 1), s));
+  KZ_TRY(graph_alloc(g, &g->d_blocks, (size_t)std::max(nb, 1), s));
   KZ_TRY(graph_alloc(g, &g->V0, (size_t)g->ldw, s));
   KZ_TRY(graph_alloc(g, &g->V[0], (size_t)g->ldw, s));
   KZ_TRY(graph_alloc(g, &g->V[1], (size_t)g->ldw, s));
-  KZ_CUDA_TRY(cudaMemsetAsync(g->V0, 0, (size_t)g->ldw * 4, s));
-  KZ_TRY(graph_alloc(g, &g->d_blocks, (size_t)std::max(nb, 1), s));
-  if (nb) {
-    KZ_TRY(h2d(g->d_blocks, g->blocks.data(), sizeof(BlockDesc) * nb, s));
-    init_vlive_kernel<<<(nb + 255) / 256, 256, 0, s>>>(g->V0, g->d_blocks, nb, g->k);
-    KZ_CUDA_TRY(cudaGetLastError());
-  }
-  KZ_TRY(graph_alloc(g, &g->d_coff, (size_t)g->k + 1, s));
-  KZ_TRY(h2d(g->d_coff, g->coff.data(), sizeof(int32_t) * (g->k + 1), s));
-  KZ_TRY(graph_alloc(g, &g->d_rounds, (size_t)g->k, s));
-  KZ_TRY(h2d(g->d_rounds, g->rounds.data(), sizeof(int32_t) * g->k, s));
-  KZ_TRY(cta_prepare(g, s));  // block-pair offsets and class block offsets (the unit list needs them)
+  KZ_TRY(h2d(d, h.data(), sizeof(int32_t) * total, s));
+  g->d_perm = d;
+  g->d_coff = d + at_coff;
+  g->d_boff = d + at_boff;
+  g->d_rounds = d + at_rounds;
+  g->d_pair_off = d + at_poff;
+  const int most = std::max(n, g->ldw);
+  tables_kernel<<<std::max(1, std::min((most + 255) / 256, 4 * sm_count())), 256, 0, s>>>(
+      g->d_perm, g->d_coff, g->d_boff, n, k, nb, g->ldw, g->d_inv, g->d_col, g->d_cpos, g->d_blocks, g->V0);
+  return cuda_status(cudaGetLastError());
+}
+
+kz_status bitset_finish_load(kz_graph g, cudaStream_t s) {
+  const int nb = (int)g->blocks.size();
   // the half-word plane-0 test pays off when 16 members of a class almost
   // always hold a common neighbour: dense graphs
   {

@@ -286,19 +286,6 @@ static int device_smem_optin() {
 // rows and of the live words).
 size_t cta_smem_words(kz_graph g) { return 2 * ((size_t)g->n * g->ldw + (size_t)g->ldw); }
 
-kz_status cta_prepare(kz_graph g, cudaStream_t s) {
-  // prefix of the block pairs (x, y) with class(x) < class(y)
-  const int nb = (int)g->blocks.size();
-  std::vector<int32_t> poff((size_t)nb + 1, 0);
-  for (int x = 0; x < nb; x++) poff[x + 1] = poff[x] + (nb - g->boff[g->blocks[x].c + 1]);
-  KZ_TRY(graph_alloc(g, &g->d_pair_off, (size_t)nb + 1, s));
-  KZ_TRY(h2d(g->d_pair_off, poff.data(), sizeof(int32_t) * (nb + 1), s));
-  KZ_TRY(graph_alloc(g, &g->d_boff, (size_t)g->k + 1, s));
-  KZ_TRY(h2d(g->d_boff, g->boff.data(), sizeof(int32_t) * (g->k + 1), s));
-  g->n_pairs = poff[nb];
-  return KZ_OK;
-}
-
 static CtaGraph describe(kz_graph g, int64_t max_sweeps);
 
 // Descriptor of the graph for single-graph in-CTA launches (needs every

@@ -101,6 +101,7 @@ struct kz_graph_s {
   CtaGraphPtr d_cta_desc = nullptr;  // this graph's in-CTA descriptor
   int32_t *d_zero = nullptr;         // a device 0 (queue order of a single graph)
   int32_t *d_perm = nullptr;   // n
+  int32_t *d_col = nullptr;    // n: class of a relabelled vertex
   kz::BlockDesc *d_blocks = nullptr;
   kz::SweepPlan plan[3];              // work of the sweep kernels per form (full, half-word, two-plane)
   uint8_t *d_changed = nullptr;       // per unit: low byte of the sweep that last changed it
@@ -189,6 +190,8 @@ kz_status bitset_pack_edges(kz_graph g, const int32_t *d_edges, int64_t m, bool 
 // Packs a host dense bit matrix (row-major, row_words words a row), copied
 // in row chunks that overlap the packing; synchronous.
 kz_status bitset_pack_dense(kz_graph g, const uint64_t *h_bits, int64_t row_words, cudaStream_t s);
+// The layout's tables on the device (before packing), from one copy.
+kz_status bitset_upload_tables(kz_graph g, cudaStream_t s);
 kz_status bitset_finish_load(kz_graph g, cudaStream_t s);
 kz_status bitset_reset(kz_graph g, cudaStream_t s);
 kz_status bitset_kernelize(kz_graph g, const kz_options &opt, cudaStream_t s);
@@ -248,7 +251,6 @@ kz_status recheck_kernelize(kz_graph g, const kz_options &opt, int full_path, cu
 void learned_release(kz_graph g);
 
 // Whole-fixpoint-in-one-CTA kernel (kz_cta.cu).
-kz_status cta_prepare(kz_graph g, cudaStream_t s);
 kz_status cta_upload_descriptor(kz_graph g, cudaStream_t s);
 bool cta_fits_shared(kz_graph g);
 // force_mode: 1 = shared mode where it fits, 0 = global mode for every graph

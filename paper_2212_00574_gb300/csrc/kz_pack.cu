@@ -604,49 +604,32 @@ kz_status bitset_vertex_alive(kz_graph g, uint8_t *host_alive, int64_t *n_live) 
   return KZ_OK;
 }
 
-// Shared set-up of the two packers: relabelling tables on the device and the
-// row buffers, the pristine one zeroed on request.  Returns the temporaries to free after the sync.
-static kz_status pack_setup(kz_graph g, cudaStream_t s, PackArgs &a, std::vector<void *> &tmp, bool zero) {
+// Shared set-up of the two packers: the row buffers (the pristine one zeroed on
+// request) and the counters.
+static kz_status pack_setup(kz_graph g, cudaStream_t s, PackArgs &a, bool zero) {
   KZ_TRY(graph_alloc(g, &g->A0, (size_t)g->n * g->ldw, s));
   KZ_TRY(graph_alloc(g, &g->A[0], (size_t)g->n * g->ldw, s));
   KZ_TRY(graph_alloc(g, &g->A[1], (size_t)g->n * g->ldw, s));
   if (zero && g->n > 0 && g->ldw > 0)
     KZ_CUDA_TRY(cudaMemsetAsync(g->A0, 0, (size_t)g->n * g->ldw * 4, s));
-  std::vector<int32_t> col_new((size_t)g->n);
-  for (int c = 0; c < g->k; c++)
-    for (int x = g->coff[c]; x < g->coff[c + 1]; x++) col_new[x] = c;
-  // small tables of the packers: carved from the graph's chunks (one
-  // allocator call at most), released with the graph
-  int32_t *d_inv = nullptr, *d_col = nullptr, *d_coff = nullptr;
-  unsigned long long *d_cnt = nullptr;  // edges, error
-  const size_t nn = (size_t)std::max(g->n, 1);
-  KZ_TRY(graph_alloc(g, &d_inv, nn, s));
-  KZ_TRY(graph_alloc(g, &d_col, nn, s));
-  KZ_TRY(graph_alloc(g, &d_coff, (size_t)g->k + 1, s));
+  unsigned long long *d_cnt = nullptr;  // edges, error: released with the graph
   KZ_TRY(graph_alloc(g, &d_cnt, 2, s));
-  tmp.clear();
-  if (g->n) {
-    KZ_TRY(h2d(d_inv, g->inv.data(), (size_t)g->n * 4, s));
-    KZ_TRY(h2d(d_col, col_new.data(), (size_t)g->n * 4, s));
-  }
-  KZ_TRY(h2d(d_coff, g->coff.data(), ((size_t)g->k + 1) * 4, s));
   KZ_CUDA_TRY(cudaMemsetAsync(d_cnt, 0, 16, s));
   a.A = g->A0;
   a.ldw = g->ldw;
   a.k = g->k;
-  a.inv = d_inv;
-  a.col = d_col;
-  a.coff = d_coff;
+  a.inv = g->d_inv;
+  a.col = g->d_col;
+  a.coff = g->d_coff;
   a.edge_count = d_cnt;
   a.error = reinterpret_cast<int32_t *>(d_cnt + 1);
   return KZ_OK;
 }
 
-static kz_status pack_finish(kz_graph g, cudaStream_t s, PackArgs &a, std::vector<void *> &tmp) {
+static kz_status pack_finish(kz_graph g, cudaStream_t s, PackArgs &a) {
   unsigned long long h[2] = {0, 0};  // edges, error
   cudaError_t e1 = cudaMemcpyAsync(h, a.edge_count, sizeof(h), cudaMemcpyDeviceToHost, s);
   cudaError_t e2 = cudaStreamSynchronize(s);
-  tmp.clear();
   if (e1 != cudaSuccess) return cuda_status(e1);
   if (e2 != cudaSuccess) return cuda_status(e2);
   if (h[1]) return (kz_status)h[1];
@@ -657,27 +640,25 @@ static kz_status pack_finish(kz_graph g, cudaStream_t s, PackArgs &a, std::vecto
 kz_status bitset_pack_edges(kz_graph g, const int32_t *d_edges, int64_t m, bool dedup,
                             cudaStream_t s) {
   PackArgs a;
-  std::vector<void *> tmp;
-  kz_status st = pack_setup(g, s, a, tmp, true);
+  kz_status st = pack_setup(g, s, a, true);
   if (st == KZ_OK && m > 0) {
     const int threads = 256;
     const int grid = (int)std::min<int64_t>((m + threads - 1) / threads, 64 * sm_count());
     pack_edges_kernel<<<grid, threads, 0, s>>>(a, d_edges, m, dedup ? 1 : 0);
     st = cuda_status(cudaGetLastError());
   }
-  kz_status st2 = st == KZ_OK ? pack_finish(g, s, a, tmp) : KZ_OK;
+  kz_status st2 = st == KZ_OK ? pack_finish(g, s, a) : KZ_OK;
   return st != KZ_OK ? st : st2;
 }
 
 kz_status bitset_pack_dense(kz_graph g, const uint64_t *h_bits, int64_t row_words, cudaStream_t s) {
   PackArgs a;
-  std::vector<void *> tmp;
   // the tile form while one column word per caller column fits in shared
   // memory (32 rows x n bits); it writes every word, the row form the upper
   // triangle of zeroed rows, which a second kernel makes symmetric
   const size_t row = (size_t)((g->n + 31) / 32) * 4, coff = (size_t)(g->k + 1) * 4;
   const bool tiles = g->n <= kTileMaxN && 32 * row + coff <= kTileSmemBytes;
-  kz_status st = pack_setup(g, s, a, tmp, !tiles);
+  kz_status st = pack_setup(g, s, a, !tiles);
   const int64_t words = (int64_t)g->n * g->ldw;
   if (st == KZ_OK && words > 0) {
     if (row + coff > kRowSmemBytes) st = KZ_ERR_UNSUPPORTED;  // beyond the bitset budget's reach
@@ -738,7 +719,7 @@ kz_status bitset_pack_dense(kz_graph g, const uint64_t *h_bits, int64_t row_word
       if (e) cudaEventDestroy(e);
     if (d_bits) dev_free(d_bits, bytes, s);
   }
-  if (st == KZ_OK) st = pack_finish(g, s, a, tmp);
+  if (st == KZ_OK) st = pack_finish(g, s, a);
   if (st == KZ_OK && tiles) {
     g->m /= 2;  // the tile form counts both halves
     g->live_packed = true;
