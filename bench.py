@@ -62,7 +62,8 @@ KERNEL_SOURCES = {
     "bitset_persistent_kernel": ["kz_bitset.cu", "kz_rules.cuh", "kz_sweep.cuh", "kz_state.cuh"],
     "bitset_sweep_kernel": ["kz_bitset.cu", "kz_rules.cuh", "kz_sweep.cuh", "kz_state.cuh"],
     "tensor_edge_kernel": ["kz_tensor.cu", "kz_state.cuh"],
-    "sparse_triangle_kernel": ["kz_sparse.cu", "kz_state.cuh"],
+    "triangle_kernel": ["kz_sparse.cu", "kz_state.cuh"],
+    "pair_kernel": ["kz_pairs.cu", "kz_state.cuh"],
 }
 
 
@@ -379,12 +380,18 @@ def timed_steps(kz, torch, handles, run, stream, flush, steps, warmup, local, pg
             "wall_s": wall, "clocks": clk}
 
 
+def pair_form(st, args):
+    """Whether a run reported on the tensor path took the pair form in its
+    place (path AUTO, E4M3, clique size = colours)."""
+    return st["path"] == 4 and args.path == "auto" and args.tensor_precision == "fp8" and st["clique_k"] == st["k"]
+
+
 def roofline_of(kz, torch, g, st, step_ms, workload, args, dev, stream):
     """Roofline of the dominant kernel of one plain run."""
     passes = max(st["passes"], 1)
     launch_s = step_ms / passes / 1e3
-    kernel = {1: "bitset_persistent_kernel", 2: "cta_fixpoint_kernel", 3: "sparse_triangle_kernel",
-              4: "tensor_edge_kernel"}.get(st["path"], "?")
+    kernel = {1: "bitset_persistent_kernel", 2: "cta_fixpoint_kernel", 3: "triangle_kernel",
+              4: "pair_kernel" if pair_form(st, args) else "tensor_edge_kernel"}.get(st["path"], "?")
     if kernel == "bitset_persistent_kernel" and args.loop != "device":
         kernel = "bitset_sweep_kernel"
     traffic, traffic_src = measured_traffic(workload, kernel)
@@ -655,8 +662,12 @@ def run_ours(args, world, rank, local, pg):
 
     # our kernels inside one timed step: the reset kernel runs outside the
     # events; inside, the run-start kernel and one persistent launch (bitset),
-    # or per pass the expand, tensor and commit kernels (tensor)
-    per_step = {1: 2, 2: 2, 3: 1 + 4 * passes, 4: 1 + 3 * passes}.get(st["path"], 1 + passes)
+    # per pass the expand, tensor and commit kernels (tensor), or the rows,
+    # pair, commit and finish kernels and in the first two the lists (pair
+    # form); the CSR path's heavy passes take four kernels each (two are
+    # counted) and its light ones are one launch together
+    per_step = {1: 2, 2: 2, 3: 2 + 4 * min(passes, 2),
+                4: 1 + 4 * passes + min(passes, 2) if pair_form(st, args) else 1 + 3 * passes}.get(st["path"], 1 + passes)
     if rank == 0:
         tt = sorted(t["per_ms"])
         line = {

@@ -434,7 +434,7 @@ kz_status kz_kernelize(kz_graph g, const kz_options *opt, void *stream) {
   if (o.dominance && (o.schedule != KZ_SCHED_PLAIN || !g->has_bitset)) return KZ_ERR_UNSUPPORTED;
   if (o.schedule == KZ_SCHED_LEARNED) {
     // learned worklist rounds on the bitset rows, certified by full passes of
-    // the path AUTO would take (the bitset sweep or the tensor form)
+    // the path AUTO would take (the bitset sweep or the pair form)
     if (!g->has_bitset || !g->model) return KZ_ERR_UNSUPPORTED;
     if (o.path != KZ_PATH_AUTO && o.path != KZ_PATH_BITSET && o.path != KZ_PATH_TENSOR) return KZ_ERR_UNSUPPORTED;
     const int full = full_pass_path(g, o);

@@ -10,7 +10,7 @@
 // result is the unique greatest fixpoint.
 //
 // Round structure of a learned kernelization (bitset rows):
-//   1. full passes (the multi-CTA sweep or the tensor form) while the
+//   1. full passes (the multi-CTA sweep, pair form or tensor form) while the
 //      cascade is heavy: as long as the last pass deleted so many edges that
 //      the frontier they leave would cost more to test than a full pass;
 //   2. learned rounds: per-vertex statistics of the live graph (degree,
@@ -1488,8 +1488,8 @@ kz_status learned_kernelize(kz_graph g, const kz_options &opt, int full_path, cu
   }
 }
 
-// Dense support schedule: the first sweep is a full pass (the bitset sweep
-// or the tensor form); every later sweep either re-checks only the (pair,
+// Dense support schedule: the first sweep is a full pass (the bitset sweep,
+// the pair form or the tensor form); every later sweep either re-checks only the (pair,
 // class) combinations the previous sweep's deletions touched
 // (recheck_kernel, with the vertex rule on the current rows) or, when that
 // would cost more, is a full pass.  Both compute the same Jacobi sweep, so
