@@ -323,19 +323,19 @@ __global__ void __launch_bounds__(256) lists_kernel(const uint32_t *__restrict__
 // random and one conflict-free 4-byte shared load (about 4.5 wavefronts for 32
 // tests) whatever the class length, where pair_kernel reads W words.  Witnesses
 // live as long as a run's lists do: a deleted edge's entry becomes padding, and
-// once three tenths of the listed edges are gone the lists are built anew with
-// every hint at word 0.
+// once three tenths of the listed edges are gone the lists are built anew, and
+// the hints with them.
 //
 // A job is one class, one tile of u's (all its words of the class staged) and
 // a range of v blocks; a warp holds its block's words transposed, [word][lane].
 // Bound by shared-memory wavefronts (the random word of u above all) and by
 // the 2 bytes of list and 1 of hint a test reads.  Measured at n = 32768,
-// k = 24, p = 0.07: 2.9 ms the first pass with hints, 2.1 ms the fiftieth, where
-// pair_kernel takes 4.6; the pass that finds the hints takes 16 (every test
-// searches), so a run of 52 passes goes from 244 to 144 ms, one of 18 at
-// n = 16384 from 17.2 to 13.8, and runs of 10 gain 3 to 5%.  Runs of two passes,
-// the common kind, keep pair_kernel.  Padding tested as a row of ones instead
-// of masked: 156; list rows of four entries: 155.
+// k = 24, p = 0.07: 2.9 ms the second pass with hints, 2.1 ms the fiftieth, where
+// pair_kernel takes 4.6; the first, which finds the hints, takes 12.6 (16 when
+// every test went to the search).  A run of 52 passes goes from 244 to 141 ms,
+// one of 18 at n = 16384 from 17.2 to 12.4, one of 10 at n = 9001 from 3.3 to
+// 2.75.  Runs of two passes, the common kind, keep pair_kernel.  Padding tested
+// as a row of ones instead of masked: 8% slower; list rows of four entries: 8%.
 // ---------------------------------------------------------------------------
 
 constexpr int kHintQueue = 12;
@@ -365,21 +365,25 @@ __device__ __forceinline__ uint32_t lds32(uint32_t addr) {
   return v;
 }
 
-// The queued tests of the warp's lanes, searched over the whole class: a new
-// hint, or a failing edge.
+// The queued tests of the warp's lanes, searched over the class from its
+// 16-byte chunk `from` on: a new hint, or a failing edge.
 static __device__ __noinline__ void search_class(const HintArgs &p, const uint32_t *queue, int stride, int cnt,
                                                  const BlockDesc *tile, uint32_t rows_addr, uint32_t vt_addr, int c,
-                                                 uint32_t first, int v, const BlockDesc Y, unsigned int &fails) {
+                                                 uint32_t first, int from, int v, const BlockDesc Y,
+                                                 unsigned int &fails) {
   const int lane = threadIdx.x & 31;
   const int quads = p.Rp >> 2;
   // every lane walks its own queue, one 16-byte chunk a step, so lanes with
   // short searches move on to their next test
   uint32_t e = 0, row = 0;
-  for (int i = -1, q = 0;;) {
-    if (q == 0) {
+  bool next = true;
+  for (int i = -1, q = from;;) {
+    if (next) {
       if (++i >= cnt) break;
       e = queue[i * stride];
       row = rows_addr + (e & 0xffffu) * (uint32_t)p.Rp * 4u;
+      q = from;
+      next = false;
     }
     const uint4 a = lds128(row + 16 * q);
     const uint32_t vw = vt_addr + 512 * q;
@@ -401,12 +405,15 @@ static __device__ __noinline__ void search_class(const HintArgs &p, const uint32
       atomicOr(&p.Edel[(int64_t)u * p.ldw + Y.r * p.k + Y.c], 1u << lane);
       fails += (old & bu) ? 0u : 1u;
     }
-    q = 0;
+    next = true;
   }
   __syncwarp();
 }
 
-template <int WARPS>
+// FRESH: the lists are new and have no hints.  A test then looks at the first
+// four words (one 16-byte load of u's row, v's words in registers), which find
+// most of the witnesses, and the hints are written as the list is walked.
+template <int WARPS, bool FRESH>
 __global__ void __launch_bounds__(32 * WARPS, 1) hint_kernel(const __grid_constant__ HintArgs p) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ BlockDesc s_tile[kTileBlocks];
@@ -471,7 +478,7 @@ __global__ void __launch_bounds__(32 * WARPS, 1) hint_kernel(const __grid_consta
       }
       if (n2 == 0) continue;
       const uint32_t *lp = p.lists + (int64_t)first * 32 + lane;
-      const uint16_t *hp = p.hints + (c * p.hint_rows + (int64_t)first) * 32 + lane;
+      uint16_t *hp = p.hints + (c * p.hint_rows + (int64_t)first) * 32 + lane;
       const uint32_t pads = (uint32_t)tile_rows * 0x10001u;
       // list rows and hints kHintAhead steps (of two rows) ahead
       uint32_t le[kHintAhead][2], lh[kHintAhead][2];
@@ -481,7 +488,7 @@ __global__ void __launch_bounds__(32 * WARPS, 1) hint_kernel(const __grid_consta
         for (int r = 0; r < 2; r++) {
           const int i = 2 * d + r;
           le[d][r] = i < n2 ? lp[i * 32] : pads;
-          lh[d][r] = i < n2 ? hp[i * 32] : 0u;
+          if constexpr (!FRESH) lh[d][r] = i < n2 ? hp[i * 32] : 0u;
         }
       const int v = Yc.base + min(lane, Yc.size - 1);
       const uint4 *vrow = reinterpret_cast<const uint4 *>(cmc + (int64_t)v * Rp);
@@ -495,41 +502,62 @@ __global__ void __launch_bounds__(32 * WARPS, 1) hint_kernel(const __grid_consta
         vt[128 * q + 96] = x.w;
       }
       __syncwarp();
+      uint4 v4 = make_uint4(0u, 0u, 0u, 0u);
+      if constexpr (FRESH) v4 = make_uint4(vt[0], vt[32], vt[64], vt[96]);
       int cnt = 0;
       for (int i0 = 0; i0 < n2; i0 += 2 * kHintAhead) {
 #pragma unroll
         for (int d = 0; d < kHintAhead; d++) {
           const int i = i0 + 2 * d;
           const uint32_t e[4] = {le[d][0] & 0xffffu, le[d][0] >> 16, le[d][1] & 0xffffu, le[d][1] >> 16};
-          const uint32_t h[4] = {lh[d][0] & 0xffu, lh[d][0] >> 8, lh[d][1] & 0xffu, lh[d][1] >> 8};
+          uint32_t h[4] = {0u, 0u, 0u, 0u};
+          if constexpr (!FRESH) {
+            h[0] = lh[d][0] & 0xffu;
+            h[1] = lh[d][0] >> 8;
+            h[2] = lh[d][1] & 0xffu;
+            h[3] = lh[d][1] >> 8;
+          }
 #pragma unroll
           for (int r = 0; r < 2; r++) {
             const int in = i + 2 * kHintAhead + r;
             le[d][r] = in < n2 ? lp[in * 32] : pads;
-            lh[d][r] = in < n2 ? hp[in * 32] : 0u;
+            if constexpr (!FRESH) lh[d][r] = in < n2 ? hp[in * 32] : 0u;
           }
           bool miss[4];
           bool any = false;
 #pragma unroll
           for (int x = 0; x < 4; x++) {
-            const uint32_t wu = lds32(rows_addr + mad(min(e[x], last_row), row_bytes, h[x] * 4u));
-            const uint32_t wv = lds32(vt_addr + h[x] * 128u);
-            miss[x] = (wu & wv) == 0u && e[x] <= last_row;
+            if constexpr (FRESH) {
+              const uint4 a = lds128(mad(min(e[x], last_row), row_bytes, rows_addr));
+              const uint32_t m0 = a.x & v4.x, m1 = a.y & v4.y, m2 = a.z & v4.z;
+              miss[x] = (m0 | m1 | m2 | (a.w & v4.w)) == 0u && e[x] <= last_row;
+              h[x] = m0 ? 0u : m1 ? 1u : m2 ? 2u : 3u;
+            } else {
+              const uint32_t wu = lds32(rows_addr + mad(min(e[x], last_row), row_bytes, h[x] * 4u));
+              const uint32_t wv = lds32(vt_addr + h[x] * 128u);
+              miss[x] = (wu & wv) == 0u && e[x] <= last_row;
+            }
             any |= miss[x];
+          }
+          if constexpr (FRESH) {
+            // (a queued test's hint is replaced when its search ends)
+            if (i < n2) hp[i * 32] = (uint16_t)(h[0] | h[1] << 8);
+            if (i + 1 < n2) hp[(i + 1) * 32] = (uint16_t)(h[2] | h[3] << 8);
           }
           if (__any_sync(0xffffffffu, any)) {
 #pragma unroll
             for (int x = 0; x < 4; x++)
               if (miss[x]) queue[cnt++ * (32 * WARPS)] = e[x] | (uint32_t)(2 * i + x) << 16;
             if (__any_sync(0xffffffffu, cnt > kHintQueue - 4)) {
-              search_class(p, queue, 32 * WARPS, cnt, s_tile, rows_addr, vt_addr, c, first, v, Yc, fails);
+              search_class(p, queue, 32 * WARPS, cnt, s_tile, rows_addr, vt_addr, c, first, FRESH ? 1 : 0, v, Yc,
+                           fails);
               cnt = 0;
             }
           }
         }
       }
       if (__any_sync(0xffffffffu, cnt > 0))
-        search_class(p, queue, 32 * WARPS, cnt, s_tile, rows_addr, vt_addr, c, first, v, Yc, fails);
+        search_class(p, queue, 32 * WARPS, cnt, s_tile, rows_addr, vt_addr, c, first, FRESH ? 1 : 0, v, Yc, fails);
     }
   }
   fails = __reduce_add_sync(0xffffffffu, fails);
@@ -765,6 +793,12 @@ static kz_status pairs_buffers(kz_graph g, cudaStream_t s) {
 constexpr int kHintMinWords = 12, kHintMaxWords = 255;
 constexpr size_t kHintBudgetBytes = size_t(8) << 30;
 
+typedef void (*HintFn)(const HintArgs);
+static HintFn hint_fn(int warps, bool fresh) {
+  if (warps == 16) return fresh ? hint_kernel<16, true> : hint_kernel<16, false>;
+  return fresh ? hint_kernel<8, true> : hint_kernel<8, false>;
+}
+
 static kz_status hint_buffers(kz_graph g, PairBufs &b, cudaStream_t s) {
   if (b.hint_mem || b.hint_off) return KZ_OK;
   b.hint_off = true;
@@ -803,8 +837,9 @@ static kz_status hint_buffers(kz_graph g, PairBufs &b, cudaStream_t s) {
   KZ_CUDA_TRY(cudaMemcpyAsync(b.hint_jobs, b.hint_jobs_host.data(), sizeof(int2) * b.n_hint_jobs,
                               cudaMemcpyHostToDevice, s));
   for (int w : {8, 16})
-    KZ_CUDA_TRY(cudaFuncSetAttribute(w == 8 ? (const void *)hint_kernel<8> : (const void *)hint_kernel<16>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHintSmem));
+    for (bool fresh : {false, true})
+      KZ_CUDA_TRY(cudaFuncSetAttribute((const void *)hint_fn(w, fresh), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kHintSmem));
   b.hint_off = false;
   return KZ_OK;
 }
@@ -853,6 +888,7 @@ static kz_status pairs_pass(kz_graph g, int cur, bool hints, cudaStream_t s, int
     hinted = !b.hint_off;
   }
   long long known = -1;
+  bool fresh = false;
   if (hinted) {
     if (b.hint_listed > 0 && b.live >= kHintRebuild * b.hint_listed) {
       known = (long long)b.live;
@@ -860,7 +896,7 @@ static kz_status pairs_pass(kz_graph g, int cur, bool hints, cudaStream_t s, int
       KZ_CUDA_TRY(cudaMemsetAsync(b.counts + 3, 0, 8, s));
       lists_kernel<true><<<16 * sms, 256, 0, s>>>(b.cm, b.Rp, b.pos, g->d_blocks, g->d_boff, nb, b.hint_tiles,
                                                   b.hint_tile, b.hint_refs, b.hint_lists, b.counts + 3, b.counts + 1);
-      KZ_CUDA_TRY(cudaMemsetAsync(b.hints, 0, (size_t)b.hint_rows * 64 * g->k, s));
+      fresh = true;
       b.hint_listed = b.live;
     }
     HintArgs h;
@@ -884,8 +920,7 @@ static kz_status pairs_pass(kz_graph g, int cur, bool hints, cudaStream_t s, int
     h.queue = b.queue;
     const size_t smem = (size_t)b.hint_tile * b.Rp * 128 + (size_t)b.hint_warps * (b.Rp * 128 + kHintQueue * 128);
     const int grid = (int)std::min<int64_t>((int64_t)b.n_hint_jobs * g->k, sms);
-    if (b.hint_warps == 16) hint_kernel<16><<<grid, 512, smem, s>>>(h);
-    else hint_kernel<8><<<grid, 256, smem, s>>>(h);
+    hint_fn(b.hint_warps, fresh)<<<grid, 32 * b.hint_warps, smem, s>>>(h);
   } else if (b.n_jobs > 0) {
     lists_kernel<true><<<16 * sms, 256, 0, s>>>(b.cm, b.Rp, b.pos, g->d_blocks, g->d_boff, nb, b.n_tiles,
                                                 kTileBlocks, b.refs, b.lists, b.counts + 3, b.counts + 1);
