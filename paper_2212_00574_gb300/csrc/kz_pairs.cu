@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(256) lists_kernel(const uint32_t *__restrict__
 }
 
 // ---------------------------------------------------------------------------
-// Passes after the first of a run: every test remembers a witness.
+// Passes from the third of a run on: every test remembers a witness.
 //
 // hint[class][list row][lane] names, for both entries, the word of the class
 // in which the pair last shared a bit.  A pass looks at that one word of both
