@@ -1044,14 +1044,10 @@ __global__ void __launch_bounds__(kFetchThreads) write_live_edges_kernel(const u
 
 // The flags are counted and the survivors gathered on the device, so only
 // they travel (a copy of every edge and flag, and a host scan, took 7.3 ms
-// for 5.9M edges).
-kz_status sparse_fetch(kz_graph g, uint8_t *vertex_alive, int32_t *edges_out, int64_t cap, int64_t *m_live) {
+// for 5.9M edges).  KZ_ERR_OOM when the allocator refuses the lists' memory.
+static kz_status fetch_gathered(kz_graph g, uint8_t *vertex_alive, int32_t *edges_out, int64_t cap, int64_t *m_live) {
   const int64_t m = g->m;
   cudaStream_t s = g->stream;
-  *m_live = 0;
-  if (vertex_alive && g->n)
-    KZ_CUDA_TRY(cudaMemcpyAsync(vertex_alive, g->sp_vlive, (size_t)g->n, cudaMemcpyDeviceToHost, s));
-  if (m == 0) return cuda_status(cudaStreamSynchronize(s));
   const int64_t chunks = (m + kFetchChunk - 1) / kFetchChunk;
   if (chunks > INT32_MAX) return KZ_ERR_UNSUPPORTED;
   // counts, offsets (and the total), partial sums of the scan
@@ -1066,7 +1062,11 @@ kz_status sparse_fetch(kz_graph g, uint8_t *vertex_alive, int32_t *edges_out, in
   count_live_edges_kernel<<<(unsigned)chunks, kFetchThreads, 0, s>>>(g->sp_elive, m, counts);
   kz_status st = scan_counts(counts, chunks, offset, sums, offset + chunks + 1, s);
   if (st == KZ_OK) st = cuda_status(cudaMemcpyAsync(m_live, offset + chunks, 8, cudaMemcpyDeviceToHost, s));
-  if (st == KZ_OK) st = cuda_status(cudaStreamSynchronize(s));
+  if (st == KZ_OK && vertex_alive && g->n)
+    st = cuda_status(cudaMemcpyAsync(vertex_alive, g->sp_vlive, (size_t)g->n, cudaMemcpyDeviceToHost, s));
+  // (also after a failure: no copy into the caller's memory may outlive the call)
+  kz_status waited = cuda_status(cudaStreamSynchronize(s));
+  if (st == KZ_OK) st = waited;
   const int64_t take = edges_out ? std::min<int64_t>(*m_live, cap) : 0;
   if (st == KZ_OK && take > 0) {
     out_bytes = (size_t)take * sizeof(int2);
@@ -1078,10 +1078,55 @@ kz_status sparse_fetch(kz_graph g, uint8_t *vertex_alive, int32_t *edges_out, in
       st = cuda_status(cudaGetLastError());
     }
     if (st == KZ_OK) st = cuda_status(cudaMemcpyAsync(edges_out, d_out, out_bytes, cudaMemcpyDeviceToHost, s));
-    if (st == KZ_OK) st = cuda_status(cudaStreamSynchronize(s));
+    waited = cuda_status(cudaStreamSynchronize(s));
+    if (st == KZ_OK) st = waited;
   }
   if (d_out) dev_free(d_out, out_bytes, s);
   dev_free(tmp, bytes, s);
+  return st;
+}
+
+// The same without device memory: every edge and flag to the host, and a scan
+// there.
+static kz_status fetch_scanned(kz_graph g, uint8_t *vertex_alive, int32_t *edges_out, int64_t cap, int64_t *m_live) {
+  const size_t m = (size_t)g->m;
+  cudaStream_t s = g->stream;
+  std::vector<int32_t> ends;
+  std::vector<uint8_t> live;
+  try {
+    ends.resize(2 * m);
+    live.resize(m);
+  } catch (...) {
+    return KZ_ERR_OOM;
+  }
+  kz_status st = KZ_OK;
+  const auto copy = [&](void *dst, const void *src, size_t bytes) {
+    if (st == KZ_OK && bytes) st = cuda_status(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s));
+  };
+  copy(ends.data(), g->sp_eu, 4 * m);
+  copy(ends.data() + m, g->sp_ev, 4 * m);
+  copy(live.data(), g->sp_elive, m);
+  if (vertex_alive) copy(vertex_alive, g->sp_vlive, (size_t)g->n);
+  const kz_status waited = cuda_status(cudaStreamSynchronize(s));
+  if (st == KZ_OK) st = waited;
+  if (st != KZ_OK) return st;
+  int64_t cnt = 0;
+  for (size_t e = 0; e < m; e++) {
+    if (!live[e]) continue;
+    if (cnt < cap && edges_out) {
+      edges_out[2 * cnt] = ends[e];
+      edges_out[2 * cnt + 1] = ends[m + e];
+    }
+    cnt++;
+  }
+  *m_live = cnt;
+  return KZ_OK;
+}
+
+kz_status sparse_fetch(kz_graph g, uint8_t *vertex_alive, int32_t *edges_out, int64_t cap, int64_t *m_live) {
+  *m_live = 0;
+  kz_status st = g->m > 0 ? fetch_gathered(g, vertex_alive, edges_out, cap, m_live) : KZ_ERR_OOM;
+  if (st == KZ_ERR_OOM) st = fetch_scanned(g, vertex_alive, edges_out, cap, m_live);
   return st;
 }
 
