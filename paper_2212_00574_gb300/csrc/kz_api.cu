@@ -386,14 +386,22 @@ static int auto_path(kz_graph g) {
   return tensor_preferred(g) ? KZ_PATH_TENSOR : KZ_PATH_BITSET;
 }
 
-// AUTO runs the pair form of the passes (kz_pairs.cu) wherever the table says
-// TENSOR: it gives the same sweeps and counts and was faster at every point
-// measured there (n = 4500 to 32768, density 0.07 to 0.2: 0.13 against 0.16 ms
-// a pass to 2.7 against 14.3 ms).  It takes the thesis's rules only, so a
-// clique size below k and BF16 operands stay on the tensor cores.  Such a run
-// reports KZ_PATH_TENSOR, as the table's choice.
+// AUTO runs the pair form of the passes (kz_pairs.cu) where the table says
+// TENSOR, except on the smallest graphs of the table's region when an edge
+// expects many common neighbours a class.  It gives the same sweeps and counts.
+// Times to the fixpoint over the tensor form's, 1038 k-partite graphs of the
+// region with n = 3080 to 24000, k = 3 to 64, p = 0.03 to 0.245: 0.14 to 0.91
+// from n = 6000 on (n = 32768: 2.7 against 14.3 ms a pass), 0.47 to 1.05 down to
+// n = 4400.  Below, its lists and few jobs can take as long as the tensor form's
+// whole count: where it is left out here, 0.80 to 1.34, mean 1.07 (n = 3080, k =
+// 12, p = 0.2: 1.18); where it is kept, 0.62 to 1.13, mean 0.77 (p = 0.1: 0.78).
+// It takes the thesis's rules only, so a clique size below k and BF16 operands
+// stay on the tensor cores.  Such a run reports KZ_PATH_TENSOR, as the table's
+// choice.
 static bool pairs_stand_in(kz_graph g, const kz_options &o) {
-  return o.path == KZ_PATH_AUTO && o.tensor_precision == 0 && g->slack == 0;
+  if (o.path != KZ_PATH_AUTO || o.tensor_precision != 0 || g->slack != 0) return false;
+  const double common = g->density * g->density * g->n / g->k;  // an edge's common neighbours in a class
+  return g->n >= 4400 || common < (g->n < 4200 ? 7.0 : 30.0);
 }
 
 // The full passes of the learned and support schedules.
