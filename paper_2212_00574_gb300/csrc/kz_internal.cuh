@@ -283,6 +283,11 @@ struct SparseReport {
 kz_status sparse_begin(kz_graph g, int64_t max_sweeps, cudaStream_t s);
 kz_status sparse_one_pass(kz_graph g, int64_t max_sweeps, cudaStream_t s, SparseReport *out);
 kz_status sparse_finish_small(kz_graph g, int64_t max_sweeps, const SparseReport &r, cudaStream_t s, bool *done);
+// For the support schedule: the shares of live and of failing edges, from a
+// sample taken at a run's start, and whether the whole graph fits the bitset
+// remnant.
+kz_status sparse_sample(kz_graph g, cudaStream_t s, double *live, double *failing);
+bool sparse_fits_small(kz_graph g);
 // Working and oriented rows of the live edges; their triangles into per-class
 // edge counts (support schedule).
 kz_status sparse_orient_live(kz_graph g, cudaStream_t s);

@@ -14,7 +14,8 @@
 //
 // The heavy sweeps at a run's start (more than a quarter of the live edges
 // deleted) are plain passes, and a remnant small enough for bitset rows ends
-// there; otherwise the counts are built and from then on, sweep t:
+// there; once a sweep is light, or when a sample says that the first will be,
+// the counts are built and from then on, sweep t:
 //   1. rule: every dirty element (its counts changed in the last update; all
 //      live elements after a recount) is tested on the counts of S_t; the
 //      failing edges are listed;
@@ -307,9 +308,17 @@ kz_status sparse_kernelize_support(kz_graph g, const kz_options &opt, cudaStream
   KZ_TRY(support_alloc(g, s, b));
   KZ_TRY(sparse_begin(g, max_sweeps, s));
   if (g->n == 0) return KZ_OK;
-  // heavy sweeps as plain passes; a remnant that fits bitset rows ends there
+  // heavy sweeps as plain passes; a remnant that fits bitset rows ends there.  A
+  // first sweep that will be light has its triangles counted at once, where a
+  // plain pass before the counts would have them enumerated twice (n = 4500, k =
+  // 8, p = 0.1: 3.5 ms so, 1.9 now; n = 200,000, mean degree 60, a heavy first
+  // sweep: 2.24 and 2.27 with the reset and the fetch).  A sample of the edges tells.
   int64_t live_edges = 0;
-  for (;;) {
+  double live = 0.0, failing = 0.0;
+  if (!sparse_fits_small(g)) KZ_TRY(sparse_sample(g, s, &live, &failing));
+  const bool light = live > 0.0 && failing * kRecountShareInv <= 1.0;
+  if (light) live_edges = (int64_t)(live * (double)g->m);
+  while (!light) {
     SparseReport r;
     KZ_TRY(sparse_one_pass(g, max_sweeps, s, &r));
     if (!r.cont) return KZ_OK;
