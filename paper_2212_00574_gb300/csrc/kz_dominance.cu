@@ -337,19 +337,48 @@ static int sms_d() {
   return sms > 0 ? sms : 1;
 }
 
+// Runs `make`; when it fails, what it took from the handle's memory goes back.
+template <class Make>
+static kz_status all_or_none(kz_graph g, cudaStream_t s, Make make) {
+  const GraphMark mark = graph_mark(g);
+  const kz_status st = make();
+  if (st != KZ_OK) graph_rollback(g, mark, s);
+  return st;
+}
+
+static kz_status vertex_buffers(kz_graph g, cudaStream_t s) {
+  if (g->dominance_bufs) return KZ_OK;
+  DominanceBufs b;
+  KZ_TRY(all_or_none(g, s, [&]() -> kz_status {
+    KZ_TRY(graph_alloc(g, &b.pos, (size_t)g->n, s));
+    KZ_TRY(graph_alloc(g, &b.deg, (size_t)g->n, s));
+    KZ_TRY(graph_alloc(g, &b.D, (size_t)g->ldw, s));
+    KZ_TRY(graph_alloc(g, &b.count, 1, s));
+    dom::position_kernel<<<4 * sms_d(), 256, 0, s>>>(g->n, g->k, g->d_coff, b.pos);
+    return cuda_status(cudaGetLastError());
+  }));
+  g->dominance_bufs = new DominanceBufs(b);
+  return KZ_OK;
+}
+
+static kz_status edge_buffers(kz_graph g, DominanceBufs &b, int grid, cudaStream_t s) {
+  if (b.rec) return KZ_OK;
+  DominanceBufs e = b;
+  e.scratch_warps = (int64_t)grid * (256 / 32);
+  KZ_TRY(all_or_none(g, s, [&]() -> kz_status {
+    KZ_TRY(graph_alloc(g, &e.n_rec, 1, s));
+    KZ_TRY(graph_alloc(g, &e.rec, (size_t)std::max<int64_t>(g->m, 1), s));
+    KZ_TRY(graph_alloc(g, &e.claim, (size_t)g->n, s));
+    return graph_alloc(g, &e.scratch, (size_t)(e.scratch_warps * 2 * g->ldw), s);
+  }));
+  b = e;
+  return KZ_OK;
+}
+
 kz_status dominance_round(kz_graph g, int64_t *removed, cudaStream_t s) {
   *removed = 0;
   if (g->n == 0) return KZ_OK;
-  if (!g->dominance_bufs) {
-    DominanceBufs *b = new DominanceBufs();
-    g->dominance_bufs = b;
-    KZ_TRY(graph_alloc(g, &b->pos, (size_t)g->n, s));
-    KZ_TRY(graph_alloc(g, &b->deg, (size_t)g->n, s));
-    KZ_TRY(graph_alloc(g, &b->D, (size_t)g->ldw, s));
-    KZ_TRY(graph_alloc(g, &b->count, 1, s));
-    dom::position_kernel<<<4 * sms_d(), 256, 0, s>>>(g->n, g->k, g->d_coff, b->pos);
-    KZ_CUDA_TRY(cudaGetLastError());
-  }
+  KZ_TRY(vertex_buffers(g, s));
   DominanceBufs &b = *static_cast<DominanceBufs *>(g->dominance_bufs);
   int32_t cur = 0;
   KZ_CUDA_TRY(cudaMemcpyAsync(&cur, &g->st->cur, 4, cudaMemcpyDeviceToHost, s));
@@ -376,26 +405,11 @@ constexpr int kEdgeDomBlocksPerSm = 4;
 kz_status edge_dominance_round(kz_graph g, int64_t *removed, cudaStream_t s) {
   *removed = 0;
   if (g->n == 0) return KZ_OK;
-  if (!g->dominance_bufs) {
-    DominanceBufs *b = new DominanceBufs();
-    g->dominance_bufs = b;
-    KZ_TRY(graph_alloc(g, &b->pos, (size_t)g->n, s));
-    KZ_TRY(graph_alloc(g, &b->deg, (size_t)g->n, s));
-    KZ_TRY(graph_alloc(g, &b->D, (size_t)g->ldw, s));
-    KZ_TRY(graph_alloc(g, &b->count, 1, s));
-    dom::position_kernel<<<4 * sms_d(), 256, 0, s>>>(g->n, g->k, g->d_coff, b->pos);
-    KZ_CUDA_TRY(cudaGetLastError());
-  }
+  KZ_TRY(vertex_buffers(g, s));
   DominanceBufs &b = *static_cast<DominanceBufs *>(g->dominance_bufs);
   const int sms = sms_d();
   const int grid = kEdgeDomBlocksPerSm * sms;
-  if (!b.rec) {
-    b.scratch_warps = (int64_t)grid * (256 / 32);
-    KZ_TRY(graph_alloc(g, &b.n_rec, 1, s));
-    KZ_TRY(graph_alloc(g, &b.rec, (size_t)std::max<int64_t>(g->m, 1), s));
-    KZ_TRY(graph_alloc(g, &b.claim, (size_t)g->n, s));
-    KZ_TRY(graph_alloc(g, &b.scratch, (size_t)(b.scratch_warps * 2 * g->ldw), s));
-  }
+  KZ_TRY(edge_buffers(g, b, grid, s));
   int32_t cur = 0;
   KZ_CUDA_TRY(cudaMemcpyAsync(&cur, &g->st->cur, 4, cudaMemcpyDeviceToHost, s));
   KZ_CUDA_TRY(cudaStreamSynchronize(s));

@@ -341,6 +341,25 @@ kz_status graph_alloc(kz_graph g, T **out, size_t count, cudaStream_t s) {
   return KZ_OK;
 }
 
+// A place in a handle's memory to go back to: buffers made on first use are all
+// there or, once a request was refused, none of them.
+struct GraphMark {
+  size_t allocs, arena_size, arena_used, arena_next;
+  uint8_t *arena;
+};
+
+inline GraphMark graph_mark(kz_graph g) {
+  return {g->allocs.size(), g->arena_size, g->arena_used, g->arena_next, g->arena};
+}
+
+inline void graph_rollback(kz_graph g, const GraphMark &m, cudaStream_t s) {
+  for (; g->allocs.size() > m.allocs; g->allocs.pop_back()) dev_free(g->allocs.back().p, g->allocs.back().bytes, s);
+  g->arena = m.arena;
+  g->arena_size = m.arena_size;
+  g->arena_used = m.arena_used;
+  g->arena_next = m.arena_next;
+}
+
 inline kz_status cuda_status(cudaError_t e) {
   if (e == cudaSuccess) return KZ_OK;
   if (e == cudaErrorMemoryAllocation) return KZ_ERR_OOM;

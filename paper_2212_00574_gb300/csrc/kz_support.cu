@@ -254,12 +254,7 @@ static int sms_of_device() {
   return std::max(sms, 1);
 }
 
-static kz_status support_alloc(kz_graph g, cudaStream_t s, SupportBufs *&out) {
-  out = static_cast<SupportBufs *>(g->support_bufs);
-  if (out) return KZ_OK;
-  if (support_bytes(g) > kSupportBudgetBytes) return KZ_ERR_UNSUPPORTED;
-  SupportBufs *b = new SupportBufs;
-  g->support_bufs = b;  // owned by the handle from here on (freed with it)
+static kz_status support_buffers(kz_graph g, cudaStream_t s, SupportBufs *b) {
   const size_t n = (size_t)std::max(g->n, 1), m = (size_t)std::max<int64_t>(g->m, 1), k = (size_t)g->k;
   KZ_TRY(graph_alloc(g, &b->cnt_e, m * k, s));
   KZ_TRY(graph_alloc(g, &b->cnt_v, n * k, s));
@@ -270,6 +265,22 @@ static kz_status support_alloc(kz_graph g, cudaStream_t s, SupportBufs *&out) {
   KZ_TRY(graph_alloc(g, &b->dlist, m, s));
   KZ_TRY(graph_alloc(g, &b->dcount, 4, s));
   b->bytes = support_bytes(g);
+  return KZ_OK;
+}
+
+static kz_status support_alloc(kz_graph g, cudaStream_t s, SupportBufs *&out) {
+  out = static_cast<SupportBufs *>(g->support_bufs);
+  if (out) return KZ_OK;
+  if (support_bytes(g) > kSupportBudgetBytes) return KZ_ERR_UNSUPPORTED;
+  const GraphMark mark = graph_mark(g);
+  SupportBufs *b = new SupportBufs;
+  const kz_status st = support_buffers(g, s, b);
+  if (st != KZ_OK) {
+    delete b;
+    graph_rollback(g, mark, s);
+    return st;
+  }
+  g->support_bufs = b;  // owned by the handle from here on (freed with it)
   out = b;
   return KZ_OK;
 }

@@ -1,0 +1,77 @@
+"""Requests refused one after another while a schedule makes its buffers (GPU
+only): the run returns KZ_ERR_OOM and gives back what it took, and the next run
+of the handle finds nothing half made."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+import oracle
+import paper_2212_00574_gb300 as kz
+from paper_2212_00574_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+class Refusing:
+    """Serves requests through torch's caching allocator; from the last `start`
+    on, the first `refuse` of them only (None: all)."""
+
+    def __init__(self):
+        import torch
+        self.refuse, self.count, self.live = None, 0, {}
+
+        def alloc(nbytes, stream, ctx):
+            self.count += 1
+            if self.refuse is not None and self.count > self.refuse:
+                return None
+            p = int(torch.cuda.caching_allocator_alloc(int(nbytes), 0, int(stream or 0)))
+            self.live[p] = int(nbytes)
+            return p
+
+        def free(ptr, nbytes, stream, ctx):
+            assert self.live.pop(int(ptr)) == nbytes
+            torch.cuda.caching_allocator_delete(int(ptr))
+
+        self.table = kz.kz_allocator(kz._ALLOC_FN(alloc), kz._FREE_FN(free), None)
+        assert kz._lib().kz_set_allocator(C.byref(self.table)) == kz.KZ_OK
+
+    def start(self, refuse):
+        self.refuse, self.count = refuse, 0
+
+
+@pytest.mark.parametrize("opts,dense", [({"path": "sparse", "schedule": "support"}, False),
+                                        ({"dominance": 2, "path": "bitset"}, True)])
+def test_every_request_refused_in_turn(opts, dense):
+    # beyond the bitset remnant (33 colours), so that the support counts are built
+    g = synth.tiny_random(9801, 1500, 33, 0.55, planted=True)
+    want = oracle.fixpoint(g.colour, g.get_edges(), g.k)
+    mem = Refusing()
+    try:
+        with kz.KernelGraph.from_synth(g, dense=dense) as kg:
+            mem.start(None)
+            kg.kernelize(**opts)
+            total = mem.count
+            ref_alive, ref_edges, _ = kg.fetch()
+        assert total >= 2 and not mem.live
+        if "dominance" not in opts:
+            assert np.array_equal(ref_alive, want["vlive"])
+            assert np.array_equal(ref_edges, g.get_edges()[want["elive"].astype(bool)])
+        for refuse in range(total):
+            mem.start(None)
+            with kz.KernelGraph.from_synth(g, dense=dense) as kg:
+                for _ in range(2):
+                    held = dict(mem.live)
+                    mem.start(refuse)
+                    with pytest.raises(kz.KzError) as e:
+                        kg.kernelize(**opts)
+                    assert e.value.status == kz.KZ_ERR_OOM and mem.count >= refuse + 1
+                    assert mem.live == held
+                    mem.start(None)
+                    kg.reset()
+                kg.kernelize(**opts)
+                alive, edges, _ = kg.fetch()
+                assert np.array_equal(alive, ref_alive) and np.array_equal(edges, ref_edges)
+            assert not mem.live
+    finally:
+        kz.use_default_allocator()
