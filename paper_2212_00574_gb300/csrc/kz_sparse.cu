@@ -1216,9 +1216,14 @@ static kz_status fetch_scanned(kz_graph g, uint8_t *vertex_alive, int32_t *edges
   return KZ_OK;
 }
 
+// Edges up to which everything travels to the host: the gathering takes two
+// requests, five launches and two waits, 100 us however few there are, and the
+// scan 69 us for 434 edges, 87 for 20,000, 99 for 35,000 and 173 for 120,000.
+constexpr int64_t kScanEdges = 32768;
+
 kz_status sparse_fetch(kz_graph g, uint8_t *vertex_alive, int32_t *edges_out, int64_t cap, int64_t *m_live) {
   *m_live = 0;
-  kz_status st = g->m > 0 ? fetch_gathered(g, vertex_alive, edges_out, cap, m_live) : KZ_ERR_OOM;
+  kz_status st = g->m > kScanEdges ? fetch_gathered(g, vertex_alive, edges_out, cap, m_live) : KZ_ERR_OOM;
   if (st == KZ_ERR_OOM) st = fetch_scanned(g, vertex_alive, edges_out, cap, m_live);
   return st;
 }
