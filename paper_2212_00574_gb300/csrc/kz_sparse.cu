@@ -31,6 +31,7 @@
 
 #include <algorithm>
 #include <cstddef>
+#include <type_traits>
 #include <vector>
 
 #include "kz_internal.cuh"
@@ -176,20 +177,82 @@ __global__ void vinfo_kernel(const int32_t *__restrict__ rank, const int32_t *__
 
 __device__ __forceinline__ int64_t list_size(const SparseArgs &a) { return a.list ? (int64_t)*a.n_list : a.n; }
 
-// 1. The vertex rule, one warp per vertex.
-__global__ void __launch_bounds__(256) vertex_kernel(SparseArgs a) {
-  const int lane = threadIdx.x & 31;
+// The kernels over the vertices (1, 2 and 4) give a vertex a warp.  In a pass
+// over every vertex of a graph whose mean row has fewer than kShortRow entries
+// four vertices share one, eight lanes each, and the warp takes rows of more than
+// kLongRow entries afterwards, one after another.  (Later passes are left with
+// the core, where four long rows to a warp cost more than short ones gain.)  A
+// run on 200,000 vertices, k = 3, mean degree 6: 691 us with a warp each, 559
+// so; mean degree 12: 806 and 648; power-law degrees, 300,000, mean 6: 1073 and
+// 984; 100,000, mean 20 (a warp each either way): 3330.
+constexpr int kShortRow = 16, kLongRow = 64;
+
+// The lanes of a vertex, as one of them sees them: its place among them, the
+// first one's lane, and as bits of the warp's lanes all of them and those before
+// this one.
+template <int LANES>
+struct Group {
+  static constexpr int kLanes = LANES;
+  __device__ __forceinline__ static int lane() { return threadIdx.x & (LANES - 1); }
+  __device__ __forceinline__ static int shift() { return LANES == 32 ? 0 : threadIdx.x & 32 - LANES; }
+  __device__ __forceinline__ static uint32_t mine() {
+    return LANES == 32 ? 0xffffffffu : ((1u << (LANES & 31)) - 1u) << shift();
+  }
+  __device__ __forceinline__ static uint32_t before() { return mine() & ((1u << (threadIdx.x & 31)) - 1u); }
+};
+
+// body(group, vertex, first, end) for the pass's vertices: the bounds that
+// row(vertex, first, end) gives.
+template <bool SHORT, class Row, class Body>
+__device__ __forceinline__ void over_vertices(const SparseArgs &a, Row row, Body body) {
   const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = list_size(a), sweep_no = a.st->sweeps;
+  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5, total = list_size(a);
+  const Group<32> W;
+  if constexpr (!SHORT) {
+    for (int64_t i = warp0; i < total; i += warps) {
+      const int32_t u = a.list ? a.list[i] : (int32_t)i;
+      int64_t b, e;
+      row(u, b, e);
+      body(W, u, b, e);
+    }
+  } else {
+    const Group<8> G;
+    for (int64_t i0 = 4 * warp0; i0 < total; i0 += 4 * warps) {
+      const int64_t i = i0 + (G.shift() >> 3);
+      int32_t u = 0;
+      int64_t b = 0, e = 0;
+      if (i < total) {
+        u = a.list ? a.list[i] : (int32_t)i;
+        row(u, b, e);
+        if (e - b <= kLongRow) body(G, u, b, e);
+      }
+      __syncwarp();
+      for (uint32_t left = __ballot_sync(0xffffffffu, G.lane() == 0 && e - b > kLongRow); left; left &= left - 1) {
+        const int from = __ffs(left) - 1;
+        const int32_t v = __shfl_sync(0xffffffffu, u, from);
+        body(W, v, __shfl_sync(0xffffffffu, b, from), __shfl_sync(0xffffffffu, e, from));
+        __syncwarp();
+      }
+    }
+  }
+  __syncwarp();
+}
+
+// 1. The vertex rule.
+template <bool SHORT>
+__global__ void __launch_bounds__(256) vertex_kernel(SparseArgs a) {
+  const int64_t sweep_no = a.st->sweeps;
   const int32_t *adj = a.from_input ? a.adj0 : a.adj, *eid = a.from_input ? a.eid0 : a.eid;
   unsigned long long tests = 0, dv = 0;
-  for (int64_t i = warp0; i < total; i += warps) {
-    const int32_t u = a.list ? a.list[i] : (int32_t)i;
-    const int64_t b = a.row0[u], e = b + (a.from_input ? a.row0[u + 1] - b : a.len[u]);
+  const auto row = [&](int32_t u, int64_t &b, int64_t &e) {
+    b = a.row0[u];
+    e = b + (a.from_input ? a.row0[u + 1] - b : a.len[u]);
+  };
+  over_vertices<SHORT>(a, row, [&](const auto &G, int32_t u, int64_t b, int64_t e) {
+    constexpr int L = std::decay_t<decltype(G)>::kLanes;
     const int32_t ru = a.rank[u];
     unsigned long long cm = 0;
-    for (int64_t j = b + lane; j < e; j += 32) {
+    for (int64_t j = b + G.lane(); j < e; j += L) {
       const int32_t v = adj[j];
       if (a.all_live || a.elive[eid[j]]) {
         const int2 x = a.vinfo[v];  // (another warp may set v's failing bit meanwhile: only rank and colour are read)
@@ -197,8 +260,8 @@ __global__ void __launch_bounds__(256) vertex_kernel(SparseArgs a) {
         tests += x.x > ru;
       }
     }
-    const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)cm), hi = __reduce_or_sync(0xffffffffu, (uint32_t)(cm >> 32));
-    if (lane == 0) {
+    const uint32_t lo = __reduce_or_sync(G.mine(), (uint32_t)cm), hi = __reduce_or_sync(G.mine(), (uint32_t)(cm >> 32));
+    if (G.lane() == 0) {
       cm = ((unsigned long long)hi << 32 | lo) & ~(1ull << a.col[u]);
       const bool fail = a.vlive[u] && __popcll(cm) < a.q - 1;
       a.vfail[u] = fail ? 1 : 0;
@@ -209,33 +272,35 @@ __global__ void __launch_bounds__(256) vertex_kernel(SparseArgs a) {
         a.v_sweep[u] = (int32_t)(sweep_no + 1);  // (a refused sweep's marks lie beyond the count of sweeps)
       }
     }
+  });
+  for (int o = 16; o > 0; o >>= 1) {
+    tests += __shfl_down_sync(0xffffffffu, tests, o);
+    dv += __shfl_down_sync(0xffffffffu, dv, o);
   }
-  for (int o = 16; o > 0; o >>= 1) tests += __shfl_down_sync(0xffffffffu, tests, o);
-  if (lane == 0) {
+  if ((threadIdx.x & 31) == 0) {
     if (tests) atomicAdd(&a.st->pass_tests, tests);
     if (dv) atomicAdd(&a.st->pass_dv, dv);
   }
 }
 
 // 2. Rows of passing vertices, oriented rows, work items, the next vertex
-// list; edges of failing vertices go.  One warp per vertex; the row shrinks in
-// place behind the reads.
+// list; edges of failing vertices go.  The row shrinks in place behind the
+// reads.
+template <bool SHORT>
 __global__ void __launch_bounds__(256) orient_kernel(SparseArgs a) {
-  const int lane = threadIdx.x & 31;
-  const uint32_t lt = (1u << lane) - 1u;
-  const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = list_size(a);
   const int32_t *adj = a.from_input ? a.adj0 : a.adj, *eid = a.from_input ? a.eid0 : a.eid;
   unsigned long long de = 0;
-  for (int64_t i = warp0; i < total; i += warps) {
-    const int32_t u = a.list ? a.list[i] : (int32_t)i;
-    const int64_t b = a.row0[u], end = b + (a.from_input ? a.row0[u + 1] - b : a.len[u]);
+  const auto row = [&](int32_t u, int64_t &b, int64_t &e) {
+    b = a.row0[u];
+    e = b + (a.from_input ? a.row0[u + 1] - b : a.len[u]);
+  };
+  over_vertices<SHORT>(a, row, [&](const auto &G, int32_t u, int64_t b, int64_t end) {
+    constexpr int L = std::decay_t<decltype(G)>::kLanes;
     const int32_t ru = a.rank[u];
     const bool fu = a.vfail[u] != 0;
     int32_t pl = 0, po = 0;
-    for (int64_t base = b; base < end; base += 32) {
-      const int64_t j = base + lane;
+    for (int64_t base = b; base < end; base += L) {
+      const int64_t j = base + G.lane();
       int32_t v = 0, ed = 0;
       bool keep = false, ori = false;
       if (j < end) {
@@ -253,46 +318,46 @@ __global__ void __launch_bounds__(256) orient_kernel(SparseArgs a) {
           if (up && keep) a.mask[ed] = 0ull;
         }
       }
-      const uint32_t mk = __ballot_sync(0xffffffffu, keep), mo = __ballot_sync(0xffffffffu, ori);
+      __syncwarp(G.mine());  // this step's reads precede its writes, which lie at or before them
+      const uint32_t mk = __ballot_sync(G.mine(), keep) & G.mine(), mo = __ballot_sync(G.mine(), ori) & G.mine();
       if (keep && a.apply) {
-        a.adj[b + pl + __popc(mk & lt)] = v;
-        a.eid[b + pl + __popc(mk & lt)] = ed;
+        a.adj[b + pl + __popc(mk & G.before())] = v;
+        a.eid[b + pl + __popc(mk & G.before())] = ed;
       }
       if (ori) {
-        a.oadj[b + po + __popc(mo & lt)] = v;
-        a.oeid[b + po + __popc(mo & lt)] = ed;
+        a.oadj[b + po + __popc(mo & G.before())] = v;
+        a.oeid[b + po + __popc(mo & G.before())] = ed;
       }
       pl += __popc(mk);
       po += __popc(mo);
-      __syncwarp();  // this step's reads precede the next step's writes
     }
     const bool live = a.vlive[u] != 0;
-    if (lane == 0) {
+    if (G.lane() == 0) {
       a.olen[u] = po;
       if (a.apply) {
         a.len[u] = pl;
         if (live && !fu) a.list_out[atomicAdd(a.n_out, 1u)] = u;
       }
     }
-    if (po < 2) continue;  // no triangle starts here
+    if (po < 2) return;  // no triangle starts here
     if (po <= kTableKeys) {
       const int parts = (po + kItemEdges - 1) / kItemEdges;
       unsigned int at = 0;
-      if (lane == 0) at = atomicAdd(a.n_items, (unsigned int)parts);
-      at = __shfl_sync(0xffffffffu, at, 0);
-      if (lane < parts) a.items[at + lane] = make_int2(u, lane);
+      if (G.lane() == 0) at = atomicAdd(a.n_items, (unsigned int)parts);
+      at = __shfl_sync(G.mine(), at, G.shift());
+      if (G.lane() < parts) a.items[at + G.lane()] = make_int2(u, G.lane());
     } else {
       unsigned int at = 0;
-      if (lane == 0) at = atomicAdd(a.n_big, (unsigned int)po);
-      at = __shfl_sync(0xffffffffu, at, 0);
-      for (int32_t t = lane; t < po; t += 32) {
+      if (G.lane() == 0) at = atomicAdd(a.n_big, (unsigned int)po);
+      at = __shfl_sync(G.mine(), at, G.shift());
+      for (int32_t t = G.lane(); t < po; t += L) {
         a.big_u[at + t] = u;
         a.big_i[at + t] = t;
       }
     }
-  }
+  });
   for (int o = 16; o > 0; o >>= 1) de += __shfl_down_sync(0xffffffffu, de, o);
-  if (lane == 0 && de) atomicAdd(&a.st->pass_de, de);
+  if ((threadIdx.x & 31) == 0 && de) atomicAdd(&a.st->pass_de, de);
 }
 
 // OR of bits into a mask; most repeat, so they are looked up first.
@@ -499,26 +564,24 @@ __global__ void __launch_bounds__(256) triangle_big_kernel(SparseArgs a, uint32_
 }
 
 // 4. The edge rule on the masks, over the oriented edges of passing vertices.
+template <bool SHORT>
 __global__ void __launch_bounds__(256) verdict_kernel(SparseArgs a) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = list_size(a);
   unsigned long long de = 0;
-  for (int64_t i = warp0; i < total; i += warps) {
-    const int32_t u = a.list ? a.list[i] : (int32_t)i;
-    if (a.vfail[u]) continue;
-    const int64_t b = a.row0[u], e = b + a.olen[u];
-    for (int64_t j = b + lane; j < e; j += 32) {
+  const auto row = [&](int32_t u, int64_t &b, int64_t &e) {
+    b = a.row0[u];
+    e = b + (a.vfail[u] ? 0 : a.olen[u]);
+  };
+  over_vertices<SHORT>(a, row, [&](const auto &G, int32_t, int64_t b, int64_t e) {
+    for (int64_t j = b + G.lane(); j < e; j += G.kLanes) {
       if (a.vfail[a.oadj[j]]) continue;
       const int32_t ed = a.oeid[j];
       if (__popcll(a.mask[ed]) >= a.q - 2) continue;
       de++;
       if (a.apply) a.elive[ed] = 0;
     }
-  }
+  });
   for (int o = 16; o > 0; o >>= 1) de += __shfl_down_sync(0xffffffffu, de, o);
-  if (lane == 0 && de) atomicAdd(&a.st->pass_de, de);
+  if ((threadIdx.x & 31) == 0 && de) atomicAdd(&a.st->pass_de, de);
 }
 
 // Of the edges spread over the list, one per CTA: how many are live (found[0])
@@ -938,13 +1001,16 @@ static SparseArgs sparse_args(kz_graph g, bool use_list, int in, bool apply) {
   return a;
 }
 
+static bool short_rows(kz_graph g) { return 2 * g->m < (int64_t)kShortRow * g->n; }
+
 // Working and oriented rows of the live edges, no vertex left out, with the
 // triangles' work items (support schedule).
 kz_status sparse_orient_live(kz_graph g, cudaStream_t s) {
   KZ_CUDA_TRY(cudaMemsetAsync(g->sp_vfail, 0, (size_t)std::max(g->n, 1), s));
   if (g->n) vinfo_kernel<<<std::min(8 * sms_here(), (g->n + 255) / 256), 256, 0, s>>>(g->sp_rank, g->sp_col, g->n, g->sp_vinfo);
   KZ_CUDA_TRY(cudaMemsetAsync(g->sp_ctr, 0, 4 * sizeof(unsigned int), s));
-  orient_kernel<<<16 * sms_here(), 256, 0, s>>>(sparse_args(g, false, 0, true));
+  const auto orient = short_rows(g) ? orient_kernel<true> : orient_kernel<false>;
+  orient<<<16 * sms_here(), 256, 0, s>>>(sparse_args(g, false, 0, true));
   KZ_CUDA_TRY(cudaGetLastError());
   g->sp_from_input = g->sp_all_live = false;
   return KZ_OK;
@@ -997,11 +1063,12 @@ kz_status sparse_one_pass(kz_graph g, int64_t max_sweeps, cudaStream_t s, Sparse
   const int sms = sms_here(), grid = 16 * sms;
   const bool apply = g->sp_sweeps < max_sweeps;
   const SparseArgs a = sparse_args(g, g->sp_use_list, g->sp_in, apply);
-  vertex_kernel<<<grid, 256, 0, s>>>(a);
-  orient_kernel<<<grid, 256, 0, s>>>(a);
+  const bool few = !a.list && short_rows(g);
+  (few ? vertex_kernel<true> : vertex_kernel<false>)<<<grid, 256, 0, s>>>(a);
+  (few ? orient_kernel<true> : orient_kernel<false>)<<<grid, 256, 0, s>>>(a);
   triangle_kernel<false><<<5 * sms, 32 * kTriWarps, 0, s>>>(a, nullptr);
   triangle_big_kernel<false><<<8 * sms, 256, 0, s>>>(a, nullptr);
-  verdict_kernel<<<grid, 256, 0, s>>>(a);
+  (few ? verdict_kernel<true> : verdict_kernel<false>)<<<grid, 256, 0, s>>>(a);
   sparse_finish_kernel<<<1, 1, 0, s>>>(g->st, g->sp_ctr, g->sp_in ^ 1, g->sp_report);
   KZ_CUDA_TRY(cudaGetLastError());
   long long r[4];
