@@ -821,6 +821,9 @@ static kz_status hint_buffers(kz_graph g, PairBufs &b, cudaStream_t s) {
                                                b.hint_tile, nullptr, nullptr, b.counts + 3, nullptr);
   KZ_CUDA_TRY(cudaGetLastError());
   KZ_CUDA_TRY(cudaMemcpyAsync(&rows, b.counts + 3, 8, cudaMemcpyDeviceToHost, s));
+  // the cursor goes back to zero: a pass left without hints fills pair_kernel's
+  // lists from there, which have no room for as many rows again
+  KZ_CUDA_TRY(cudaMemsetAsync(b.counts + 3, 0, 8, s));
   KZ_CUDA_TRY(cudaStreamSynchronize(s));
   const auto part = [](size_t bytes) { return (bytes + 255) & ~(size_t)255; };
   const size_t jobs = part(sizeof(int2) * b.n_hint_jobs), refs = part(sizeof(ListRef) * b.hint_tiles * nb);

@@ -75,3 +75,33 @@ def test_every_request_refused_in_turn(opts, dense):
             assert not mem.live
     finally:
         kz.use_default_allocator()
+
+
+# from the third pass on the runs of the pair form keep witnesses, in memory that
+# they ask for once a run and do without when it is refused
+@pytest.mark.parametrize("n,k,p", [(5200, 12, 0.11), (7001, 11, 0.09)])
+def test_long_cascade_without_the_witnesses_memory(n, k, p):
+    g = synth.kpartite(n, k, p, 9400 + n, planted=True)
+    kz.use_default_allocator()
+    mem = Refusing()
+    try:
+        with kz.KernelGraph.from_synth(g, dense=True) as kg:
+            kg.kernelize(path="bitset")
+            want_alive, want, want_st = kg.fetch()
+            assert want_st["passes"] >= 4
+            kg.reset().kernelize()
+            mem.start(None)
+            kg.reset().kernelize()
+            assert mem.count == 1  # the witnesses; everything else is there
+            held = dict(mem.live)
+            mem.start(0)
+            kg.reset().kernelize()
+            assert mem.count == 1 and mem.live == held  # refused
+            mem.start(None)
+            alive, edges, st = kg.fetch()
+        assert np.array_equal(alive, want_alive) and np.array_equal(edges, want)
+        for f in ("sweeps", "passes", "edge_tests", "m_live"):
+            assert st[f] == want_st[f], f
+        assert not mem.live
+    finally:
+        kz.use_default_allocator()
