@@ -404,11 +404,18 @@ static bool pairs_stand_in(kz_graph g, const kz_options &o) {
   return g->n >= 4400 || common < (g->n < 4200 ? 7.0 : 30.0);
 }
 
+// Its memory is asked for first: where the rows and lists are refused (the lists
+// of a graph with a hub in every block of vertices take twice the tensor form's
+// operands) the tensor form still runs.
+static bool pairs_run(kz_graph g, const kz_options &o) {
+  return pairs_stand_in(g, o) && pairs_buffers(g, g->stream) == KZ_OK;
+}
+
 // The full passes of the learned and support schedules.
 static int full_pass_path(kz_graph g, const kz_options &o) {
   if (o.path != KZ_PATH_AUTO) return o.path;
   if (!tensor_preferred(g)) return KZ_PATH_BITSET;
-  return pairs_stand_in(g, o) ? kFullPairs : KZ_PATH_TENSOR;
+  return pairs_run(g, o) ? kFullPairs : KZ_PATH_TENSOR;
 }
 
 static kz_status run_one(kz_graph g, const kz_options &o, int path) {
@@ -422,7 +429,7 @@ static kz_status run_one(kz_graph g, const kz_options &o, int path) {
     // only the multi-CTA sweep kernels keep the two row buffers in step
     if (path != KZ_PATH_BITSET) g->ab_synced = false;
     if (path == KZ_PATH_SMALL) KZ_TRY(cta_kernelize_one(g, o, g->stream));
-    else if (path == KZ_PATH_TENSOR && pairs_stand_in(g, o)) KZ_TRY(pairs_kernelize(g, o, g->stream));
+    else if (path == KZ_PATH_TENSOR && pairs_run(g, o)) KZ_TRY(pairs_kernelize(g, o, g->stream));
     else if (path == KZ_PATH_TENSOR) KZ_TRY(tensor_kernelize(g, o, g->stream));
     else KZ_TRY(bitset_kernelize(g, o, g->stream));
   }

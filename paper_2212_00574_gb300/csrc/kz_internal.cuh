@@ -226,6 +226,7 @@ void tensor_release(kz_graph g);
 // Pair form of the passes (kz_pairs.cu): what AUTO runs in the tensor form's
 // region.  pairs_one_pass is to tensor_one_pass as pairs_kernelize is to
 // tensor_kernelize.
+kz_status pairs_buffers(kz_graph g, cudaStream_t s);  // its rows and lists, made on first use
 kz_status pairs_kernelize(kz_graph g, const kz_options &opt, cudaStream_t s);
 kz_status pairs_one_pass(kz_graph g, cudaStream_t s, int *cont);
 void pairs_release(kz_graph g);

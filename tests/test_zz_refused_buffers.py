@@ -77,6 +77,53 @@ def test_every_request_refused_in_turn(opts, dense):
         kz.use_default_allocator()
 
 
+@pytest.mark.parametrize("opts", [{}, {"schedule": "support"}])
+def test_pair_form_refused_leaves_the_tensor_form(opts):
+    import torch
+    g = synth.kpartite(3100, 17, 0.1, 9802, planted=True)
+    with kz.KernelGraph.from_synth(g, dense=True) as kg:
+        kg.kernelize(path="bitset")
+        want_alive, want, want_st = kg.fetch()
+    once = [None]
+    asked = []
+
+    def alloc(nbytes, stream, ctx):
+        asked.append(nbytes)
+        if once[0] is not None and len(asked) == once[0] + 1:
+            return None  # this one only
+        return int(torch.cuda.caching_allocator_alloc(int(nbytes), 0, int(stream or 0)))
+
+    def free(ptr, nbytes, stream, ctx):
+        torch.cuda.caching_allocator_delete(int(ptr))
+
+    table = kz.kz_allocator(kz._ALLOC_FN(alloc), kz._FREE_FN(free), None)
+    assert kz._lib().kz_set_allocator(C.byref(table)) == kz.KZ_OK
+    operand = g.n * g.n // 2  # the tensor form's operands take more, the pair form's buffers less
+    try:
+        with kz.KernelGraph.from_synth(g, dense=True) as kg:
+            asked.clear()
+            kg.kernelize()
+            total = len(asked)
+            assert total >= 2 and max(asked) < operand
+        for refuse in range(total):
+            with kz.KernelGraph.from_synth(g, dense=True) as kg:
+                asked.clear()
+                once[0] = refuse
+                kg.kernelize(**opts)
+                once[0] = None
+                assert max(asked) >= operand
+                alive, edges, st = kg.fetch()
+                assert np.array_equal(alive, want_alive) and np.array_equal(edges, want)
+                assert st["sweeps"] == want_st["sweeps"] and st["path"] == 4
+                asked.clear()
+                kg.reset().kernelize()  # and once memory is there again, the pair form
+                assert asked and max(asked) < operand
+                alive, edges, st = kg.fetch()
+                assert np.array_equal(edges, want) and st["edge_tests"] == want_st["edge_tests"]
+    finally:
+        kz.use_default_allocator()
+
+
 # from the third pass on the runs of the pair form keep witnesses, in memory that
 # they ask for once a run and do without when it is refused
 @pytest.mark.parametrize("n,k,p", [(5200, 12, 0.11), (7001, 11, 0.09)])
