@@ -62,8 +62,9 @@ KERNEL_SOURCES = {
     "bitset_persistent_kernel": ["kz_bitset.cu", "kz_rules.cuh", "kz_sweep.cuh", "kz_state.cuh"],
     "bitset_sweep_kernel": ["kz_bitset.cu", "kz_rules.cuh", "kz_sweep.cuh", "kz_state.cuh"],
     "tensor_edge_kernel": ["kz_tensor.cu", "kz_state.cuh"],
-    "triangle_kernel": ["kz_sparse.cu", "kz_state.cuh"],
-    "pair_kernel": ["kz_pairs.cu", "kz_state.cuh"],
+    "triangle_kernel": ["kz_sparse.cu", "kz_rules.cuh", "kz_state.cuh"],
+    "pair_kernel": ["kz_pairs.cu", "kz_rules.cuh", "kz_sweep.cuh", "kz_state.cuh"],
+    "hint_kernel": ["kz_pairs.cu", "kz_rules.cuh", "kz_sweep.cuh", "kz_state.cuh"],
 }
 
 
@@ -380,10 +381,30 @@ def timed_steps(kz, torch, handles, run, stream, flush, steps, warmup, local, pg
             "wall_s": wall, "clocks": clk}
 
 
-def pair_form(st, args):
+def pair_form(g, st, args):
     """Whether a run reported on the tensor path took the pair form in its
-    place (path AUTO, E4M3, clique size = colours)."""
-    return st["path"] == 4 and args.path == "auto" and args.tensor_precision == "fp8" and st["clique_k"] == st["k"]
+    place (path AUTO, E4M3, clique size = colours; on the smallest graphs only
+    where an edge expects few common neighbours a class)."""
+    if st["path"] != 4 or args.path != "auto" or args.tensor_precision != "fp8" or st["clique_k"] != st["k"]:
+        return False
+    sizes = np.bincount(np.asarray(g.colour), minlength=g.k).astype(np.float64)
+    density = st["m"] / max((sizes.sum() ** 2 - (sizes ** 2).sum()) / 2, 1.0)
+    return g.n >= 4400 or density ** 2 * g.n / g.k < (7.0 if g.n < 4200 else 30.0)
+
+
+def form_name(kz, g, st, args):
+    """The path that ran, "pairs" where the pair form did."""
+    if pair_form(g, st, args):
+        return "pairs"
+    return {v: k for k, v in kz.PATHS.items()}.get(st["path"], str(st["path"]))
+
+
+def pair_launches(passes):
+    """Kernels of one run of the pair form: the run start, then rows, edge test,
+    commit and finish a pass, the lists in the first two, and from the third on,
+    with witnesses, the lists counted and built once (every rebuilding as edges
+    go is one more, not counted)."""
+    return 1 + 4 * passes + min(passes, 2) + (2 if passes > 2 else 0)
 
 
 def roofline_of(kz, torch, g, st, step_ms, workload, args, dev, stream):
@@ -391,7 +412,9 @@ def roofline_of(kz, torch, g, st, step_ms, workload, args, dev, stream):
     passes = max(st["passes"], 1)
     launch_s = step_ms / passes / 1e3
     kernel = {1: "bitset_persistent_kernel", 2: "cta_fixpoint_kernel", 3: "triangle_kernel",
-              4: "pair_kernel" if pair_form(st, args) else "tensor_edge_kernel"}.get(st["path"], "?")
+              4: "tensor_edge_kernel"}.get(st["path"], "?")
+    if pair_form(g, st, args):
+        kernel = "pair_kernel" if passes <= 4 else "hint_kernel"  # (witnesses from the third pass on)
     if kernel == "bitset_persistent_kernel" and args.loop != "device":
         kernel = "bitset_sweep_kernel"
     traffic, traffic_src = measured_traffic(workload, kernel)
@@ -502,7 +525,7 @@ def learned_comparison(kz, torch, graphs, stream, flush, local, args, pg, rank):
                          "speedup": p["ms"] / lr["ms"],
                          "speedup_frontier_only": p["ms"] / res["frontier"]["ms"],
                          "speedup_support": p["ms"] / res["support"]["ms"],
-                         "plain_path": {v: k for k, v in kz.PATHS.items()}.get(p["st"]["path"]),
+                         "plain_path": form_name(kz, g, p["st"], args),
                          "sweeps": {a: res[a]["st"]["sweeps"] for a in labels},
                          "passes": {a: res[a]["st"]["passes"] for a in labels},
                          "edge_tests": {a: res[a]["st"]["edge_tests"] for a in labels},
@@ -662,12 +685,11 @@ def run_ours(args, world, rank, local, pg):
 
     # our kernels inside one timed step: the reset kernel runs outside the
     # events; inside, the run-start kernel and one persistent launch (bitset),
-    # per pass the expand, tensor and commit kernels (tensor), or the rows,
-    # pair, commit and finish kernels and in the first two the lists (pair
-    # form); the CSR path's heavy passes take four kernels each (two are
-    # counted) and its light ones are one launch together
-    per_step = {1: 2, 2: 2, 3: 2 + 4 * min(passes, 2),
-                4: 1 + 4 * passes + min(passes, 2) if pair_form(st, args) else 1 + 3 * passes}.get(st["path"], 1 + passes)
+    # per pass the expand, tensor, commit and finish kernels (tensor), or those of
+    # the pair form (pair_launches); the CSR path's heavy passes take six kernels
+    # each (two passes are counted) and its light ones are one launch together
+    per_step = {1: 2, 2: 2, 3: 2 + 6 * min(passes, 2),
+                4: pair_launches(passes) if pair_form(g, st, args) else 1 + 4 * passes}.get(st["path"], 1 + passes)
     if rank == 0:
         tt = sorted(t["per_ms"])
         line = {
@@ -676,7 +698,7 @@ def run_ours(args, world, rank, local, pg):
             "scaling": "weak", "vs_baseline": None, "dtype": "u32", "data": "synthetic",
             "config": {"workload": wdesc(args), "n": g.n, "k": g.k, "m": g.m,
                        "seed": workload_seed(args.workload),
-                       "path": {v: k for k, v in kz.PATHS.items()}.get(st["path"], str(st["path"])),
+                       "path": form_name(kz, g, st, args),
                        "pass_loop": {"device": "one cooperative persistent launch", "graph": "CUDA-graph while node",
                                      "host": "host-driven"}[args.loop],
                        "passes": passes, "sweeps": st["sweeps"], "schedule": args.schedule,

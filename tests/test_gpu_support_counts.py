@@ -64,3 +64,17 @@ def test_counts_limits_reruns_and_other_paths(n, k, p):
                 alive, kept, _ = kg.fetch()
                 assert np.array_equal(alive, full["vlive"])
                 assert np.array_equal(kept, edges[full["elive"].astype(bool)])
+
+
+@pytest.mark.parametrize("n,k,p", [(200, 4, 0.3), (2000, 6, 0.1), (4050, 5, 0.055)])
+def test_sweeps_without_counts_test_what_plain_sweeps_test(n, k, p):
+    # graphs within the bitset remnant: a plain pass, then the remnant
+    g = synth.tiny_random(9700 + n, n, k, p, planted=True)
+    orc = oracle.fixpoint(g.colour, g.get_edges(), k)
+    assert orc["sweeps"] >= 2
+    with kz.KernelGraph.from_synth(g, dense=False) as kg:
+        kg.kernelize(**SUPPORT)
+        alive, kept, st = kg.fetch()
+    want_alive, want = _state(g, orc)
+    assert np.array_equal(alive, want_alive) and np.array_equal(kept, want)
+    assert [st["sweeps"], st["passes"], st["edge_tests"]] == [orc["sweeps"], orc["passes"], orc["tests"]]
