@@ -74,7 +74,6 @@ struct PairArgs {
   const uint32_t *cm;       // current rows by class: class c of row x at (c n + x) Rp
   uint32_t *Edel;           // deletion bitmap, rows x ldw (zeroed)
   const BlockDesc *blocks;
-  const int32_t *boff;      // k + 1: first block of each class
   const ListRef *refs;      // tile-major: refs[tile * nb + block]
   const uint32_t *lists;
   const int2 *jobs;         // (tile, first block of v's)
@@ -328,14 +327,18 @@ __global__ void __launch_bounds__(256) lists_kernel(const uint32_t *__restrict__
 //
 // A job is one class, one tile of u's (all its words of the class staged) and
 // a range of v blocks; a warp holds its block's words transposed, [word][lane].
-// Bound by shared-memory wavefronts (the random word of u above all) and by
-// the 2 bytes of list and 1 of hint a test reads.  Measured at n = 32768,
-// k = 24, p = 0.07: 2.9 ms the second pass with hints, 2.1 ms the fiftieth, where
-// pair_kernel takes 4.6; the first, which finds the hints, takes 12.6 (16 when
-// every test went to the search).  A run of 52 passes goes from 244 to 141 ms,
-// one of 18 at n = 16384 from 17.2 to 12.4, one of 10 at n = 9001 from 3.3 to
-// 2.75.  Runs of two passes, the common kind, keep pair_kernel.  Padding tested
-// as a row of ones instead of masked: 8% slower; list rows of four entries: 8%.
+// Bound by latency: of 16 warps an SM 3.4 an issue wait at the staging's barriers
+// and 1.9 for lists and hints; issue slots are 40% busy, the rate of shared-memory
+// wavefronts 30% (8 per 32 tests, the staging with them; n = 9001, k = 17, p =
+// 0.112, the third pass with hints).  The
+// first pass with hints, which finds them, takes 0.58 ms there (0.99 when every
+// test went to the search), the next 0.19 and the later ones 0.13, where
+// pair_kernel takes 0.22; at n = 32768, k = 24, p = 0.07 12.6, 2.9 and 2.1 ms
+// against 4.6.  Whole runs, k-partite graphs of four seeds each: n = 32768 23 to
+// 31 passes in 73 to 91 ms (on the tensor form 329 ms for 23), n = 9001 12 to 14
+// passes in 3.1 to 3.5 ms (7.1 for 14).  Runs of two passes, the common kind, keep
+// pair_kernel.  Padding tested as a row of ones instead of masked: 8% slower; list
+// rows of four entries: 8%.
 // ---------------------------------------------------------------------------
 
 constexpr int kHintQueue = 12;
@@ -868,7 +871,6 @@ static kz_status pairs_pass(kz_graph g, int cur, bool hints, cudaStream_t s, int
   a.cm = b.cm;
   a.Edel = b.Edel;
   a.blocks = g->d_blocks;
-  a.boff = g->d_boff;
   a.refs = b.refs;
   a.lists = b.lists;
   a.jobs = b.jobs;
