@@ -55,8 +55,8 @@ kz_status kz_model_get(kz_model m, float *weights);
 
 void kz_model_free(kz_model m);
 
-/* Inference on device data: X device fp32[B][16], logits device fp32[B].
- * bf16 weights, fp32 accumulation.  Asynchronous on `stream`. */
+/* Inference on device data: X device fp32[B][16] and logits device fp32[B], at
+ * any address a float may have.  bf16 weights, fp32 accumulation.  Asynchronous on `stream`. */
 kz_status kz_mlp_forward(kz_model m, const float *X, int64_t B, float *logits, void *stream);
 
 /* Mean binary cross-entropy and its gradient with respect to the fp32 master
