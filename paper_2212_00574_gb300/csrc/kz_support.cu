@@ -311,6 +311,7 @@ static kz_status support_recount(kz_graph g, SupportBufs *b, cudaStream_t s) {
 // counts yet, by a recount once it has.  (The incremental update visits every
 // triangle a deleted edge closes, with atomics on counts shared by hub edges.)
 constexpr int64_t kRecountShareInv = 4;  // one quarter
+constexpr int kSampleDegree = 8;
 
 kz_status sparse_kernelize_support(kz_graph g, const kz_options &opt, cudaStream_t s) {
   if (!g->has_csr) return KZ_ERR_UNSUPPORTED;
@@ -322,11 +323,14 @@ kz_status sparse_kernelize_support(kz_graph g, const kz_options &opt, cudaStream
   // heavy sweeps as plain passes; a remnant that fits bitset rows ends there.  A
   // first sweep that will be light has its triangles counted at once, where a
   // plain pass before the counts would have them enumerated twice (n = 4500, k =
-  // 8, p = 0.1: 3.5 ms so, 1.9 now; n = 200,000, mean degree 60, a heavy first
-  // sweep: 2.24 and 2.27 with the reset and the fetch).  A sample of the edges tells.
+  // 8, p = 0.1: 3.5 ms so, 1.9 now).  A sample of the edges tells.  It costs 35 us,
+  // so graphs of short rows, whose triangles cost little, go without (edges need
+  // k - 2 common neighbours: fewer than kSampleDegree times that many neighbours
+  // in the mean; n = 100,000, k = 12, mean degree 60: 1.97 ms, 2.00 with it).
   int64_t live_edges = 0;
   double live = 0.0, failing = 0.0;
-  if (!sparse_fits_small(g)) KZ_TRY(sparse_sample(g, s, &live, &failing));
+  if (!sparse_fits_small(g) && 2.0 * (double)g->m >= (double)kSampleDegree * (g->k - 2) * g->n)
+    KZ_TRY(sparse_sample(g, s, &live, &failing));
   const bool light = live > 0.0 && failing * kRecountShareInv <= 1.0;
   if (light) live_edges = (int64_t)(live * (double)g->m);
   while (!light) {
