@@ -337,15 +337,6 @@ static int sms_d() {
   return sms > 0 ? sms : 1;
 }
 
-// Runs `make`; when it fails, what it took from the handle's memory goes back.
-template <class Make>
-static kz_status all_or_none(kz_graph g, cudaStream_t s, Make make) {
-  const GraphMark mark = graph_mark(g);
-  const kz_status st = make();
-  if (st != KZ_OK) graph_rollback(g, mark, s);
-  return st;
-}
-
 static kz_status vertex_buffers(kz_graph g, cudaStream_t s) {
   if (g->dominance_bufs) return KZ_OK;
   DominanceBufs b;

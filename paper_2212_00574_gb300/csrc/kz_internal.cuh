@@ -361,6 +361,15 @@ inline void graph_rollback(kz_graph g, const GraphMark &m, cudaStream_t s) {
   g->arena_next = m.arena_next;
 }
 
+// Runs `make`; when it fails, what it took from the handle's memory goes back.
+template <class Make>
+kz_status all_or_none(kz_graph g, cudaStream_t s, Make make) {
+  const GraphMark mark = graph_mark(g);
+  const kz_status st = make();
+  if (st != KZ_OK) graph_rollback(g, mark, s);
+  return st;
+}
+
 inline kz_status cuda_status(cudaError_t e) {
   if (e == cudaSuccess) return KZ_OK;
   if (e == cudaErrorMemoryAllocation) return KZ_ERR_OOM;

@@ -1288,7 +1288,7 @@ kz_status learned_kernelize(kz_graph g, const kz_options &opt, int full_path, cu
   if (!g->model) return KZ_ERR_UNSUPPORTED;
   if (!g->learned_bufs) {
     LearnedBufs *b = new LearnedBufs();
-    kz_status st = ensure_bufs(g, *b, s);
+    kz_status st = all_or_none(g, s, [&] { return ensure_bufs(g, *b, s); });
     if (st != KZ_OK) {
       delete b;
       return st;
@@ -1517,7 +1517,7 @@ constexpr double kRecheckGain = 0.8;
 kz_status recheck_kernelize(kz_graph g, const kz_options &opt, int full_path, cudaStream_t s) {
   if (!g->learned_bufs) {
     LearnedBufs *b = new LearnedBufs();
-    kz_status st = ensure_bufs(g, *b, s);
+    kz_status st = all_or_none(g, s, [&] { return ensure_bufs(g, *b, s); });
     if (st != KZ_OK) {
       delete b;
       return st;
@@ -1650,7 +1650,7 @@ kz_status learned_collect(kz_graph g, int64_t per_sweep_cap, uint64_t seed, floa
   cudaStream_t s = g->stream;
   if (!g->learned_bufs) {
     LearnedBufs *b = new LearnedBufs();
-    kz_status st = ensure_bufs(g, *b, s);
+    kz_status st = all_or_none(g, s, [&] { return ensure_bufs(g, *b, s); });
     if (st != KZ_OK) {
       delete b;
       return st;

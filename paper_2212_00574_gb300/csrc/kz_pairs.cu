@@ -780,11 +780,9 @@ kz_status pairs_buffers(kz_graph g, cudaStream_t s) {
   if (g->pairs_bufs) return KZ_OK;
   PairBufs *b = new (std::nothrow) PairBufs();
   if (!b) return KZ_ERR_OOM;
-  const GraphMark mark = graph_mark(g);
-  const kz_status st = pairs_prepare(g, *b, s);
+  const kz_status st = all_or_none(g, s, [&] { return pairs_prepare(g, *b, s); });
   if (st != KZ_OK) {
     delete b;
-    graph_rollback(g, mark, s);
     return st;
   }
   b->live = (double)g->m;

@@ -272,12 +272,10 @@ static kz_status support_alloc(kz_graph g, cudaStream_t s, SupportBufs *&out) {
   out = static_cast<SupportBufs *>(g->support_bufs);
   if (out) return KZ_OK;
   if (support_bytes(g) > kSupportBudgetBytes) return KZ_ERR_UNSUPPORTED;
-  const GraphMark mark = graph_mark(g);
   SupportBufs *b = new SupportBufs;
-  const kz_status st = support_buffers(g, s, b);
+  const kz_status st = all_or_none(g, s, [&] { return support_buffers(g, s, b); });
   if (st != KZ_OK) {
     delete b;
-    graph_rollback(g, mark, s);
     return st;
   }
   g->support_bufs = b;  // owned by the handle from here on (freed with it)

@@ -741,7 +741,7 @@ static kz_status tensor_buffers(kz_graph g, bool bf16, cudaStream_t s, TensorBuf
   TensorState &ts = *static_cast<TensorState *>(g->tensor_bufs);
   if (!ts.by[bf16]) {
     TensorBufs *nb = new TensorBufs();
-    kz_status st = tensor_prepare(g, *nb, bf16, s);
+    kz_status st = all_or_none(g, s, [&] { return tensor_prepare(g, *nb, bf16, s); });
     if (st != KZ_OK) {
       delete nb;
       return st;

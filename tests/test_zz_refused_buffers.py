@@ -152,3 +152,30 @@ def test_long_cascade_without_the_witnesses_memory(n, k, p):
         assert not mem.live
     finally:
         kz.use_default_allocator()
+
+
+@pytest.mark.parametrize("opts", [{"path": "tensor"}, {"path": "tensor", "tensor_precision": 1}])
+def test_refused_runs_keep_no_memory(opts):
+    g = synth.tiny_random(9803, 2500, 9, 0.2, planted=True)
+    want = oracle.fixpoint(g.colour, g.get_edges(), g.k)
+    mem = Refusing()
+    try:
+        with kz.KernelGraph.from_synth(g, dense=True) as kg:
+            mem.start(None)
+            kg.kernelize(**opts)
+            total = mem.count
+        assert total >= 1 and not mem.live
+        with kz.KernelGraph.from_synth(g, dense=True) as kg:
+            for refuse in range(total):
+                before = dict(mem.live)
+                mem.start(refuse)
+                with pytest.raises(kz.KzError) as e:
+                    kg.kernelize(**opts)
+                assert e.value.status == kz.KZ_ERR_OOM and mem.live == before
+            mem.start(None)
+            kg.reset().kernelize(**opts)
+            alive, edges, _ = kg.fetch()
+        assert np.array_equal(alive, want["vlive"]) and np.array_equal(edges, g.get_edges()[want["elive"].astype(bool)])
+        assert not mem.live
+    finally:
+        kz.use_default_allocator()
